@@ -153,8 +153,9 @@ int syev3_batched_static_ws(const void* A_packed6, int64_t n, void* lambda, void
 /* syev3_batched_method -- syev3_batched (FP64 only) with the variants of
  * the method the paper also describes, for studying them against the
  * production path:
- *   zero_finder    : SYEV3_ZF_PRODUCTION -- the path of syev3_batched (FP32
- *                    Borges-Gragg seeds, one FP64 step and the stopping test);
+ *   zero_finder    : SYEV3_ZF_PRODUCTION -- FP32 Borges-Gragg seeds, one FP64
+ *                    step and the stopping test (syev3_batched's for graded
+ *                    matrices);
  *                    SYEV3_ZF_BORGES_GRAGG -- the Borges-Gragg iteration of
  *                    Sec. 1.4.1 in FP64 from the start of Eq. (7);
  *                    SYEV3_ZF_NEWTON -- Newton's method of Sec. 1.4.2 in FP64,

@@ -64,8 +64,15 @@ __device__ __forceinline__ unsigned hi_mag(double x) { return (unsigned)__double
 // x > 0 (x not NaN).
 __device__ __forceinline__ bool is_pos(double x) { return __double_as_longlong(x) > 0; }
 
-// x == +0 or -0.
-__device__ __forceinline__ bool is_zero(double x) { return (dbits(x) << 1) == 0; }
+// x == +0 or -0.  (On the 32-bit halves: the compiler turns the same test, or
+// the mask of mag_bits, on the 64-bit pattern back into an FP64 instruction.)
+__device__ __forceinline__ bool is_zero(double x) {
+  return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
+}
+
+// scalbn out of line: inlined, the compiler evaluates parts of the rare paths
+// that use it -- FP64 instructions -- on the common ones.
+__device__ __noinline__ double scalbn_rare(const double x, const int k) { return scalbn(x, k); }
 
 // x * 2^k by exponent arithmetic for x >= 2^-1022 in magnitude (normal) when
 // the result is normal too; otherwise scalbn.  Zero stays zero.
@@ -74,12 +81,12 @@ __device__ __forceinline__ double mul_pow2(double x, int k) {
   const int ne = ((h >> 20) & 0x7ff) + k;
   if (((h >> 20) & 0x7ff) != 0 && ne >= 1 && ne <= 2046) return __hiloint2double(h + k * (1 << 20), __double2loint(x));
   if (is_zero(x)) return x;
-  return scalbn(x, k);
+  return scalbn_rare(x, k);
 }
 
 // |x| as an unsigned integer that orders like |x| (any non-NaN x).
 __device__ __forceinline__ uint64_t mag_bits(double x) {
-  return (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  return ((uint64_t)hi_mag(x) << 32) | (unsigned)__double2loint(x);
 }
 
 // x with its sign bit XOR-ed with bit 31 of `flip` (0 or 0x80000000).

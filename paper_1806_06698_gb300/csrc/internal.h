@@ -93,6 +93,7 @@ int record_cuda_error(cudaError_t e);
 // Read and clear the __device__ status word of each translation unit
 // (synchronise the device).
 cudaError_t take_flags_f64(unsigned* flags);
+cudaError_t take_flags_f64_study(unsigned* flags);
 cudaError_t take_flags_f32(unsigned* flags);
 cudaError_t take_flags_bwd(unsigned* flags);
 

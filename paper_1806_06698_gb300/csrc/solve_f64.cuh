@@ -349,12 +349,11 @@ struct Lane {
   int cls;
 };
 
-// Phase A: pre-scale, Sec. 1 arrow reduction, Sec. 1.1 classification.
-// kEispack selects the EISPACK-style deflation test of Sec. 1.1 (the form
-// the paper starts from) instead of the simplified one it adopts.
-template <bool kEispack = false>
-__device__ __forceinline__ Lane make_lane(const double a_in[6]) {
-  Lane L;
+// Exact power-of-two pre-scale: a = a_in 2^-e with the largest entry in
+// [0.5, 1).  When every entry is zero or stays normal, by exponent
+// arithmetic; otherwise (subnormal results or inputs, huge entries) by
+// scalbn.  False when an entry is not finite (a and e are then not set).
+__device__ __forceinline__ bool prescale(const double a_in[6], double a[6], int& e) {
   int E = 0;
   bool finite = true;
 #pragma unroll
@@ -363,35 +362,42 @@ __device__ __forceinline__ Lane make_lane(const double a_in[6]) {
     finite &= (ex != 0x7ff);
     E = max(E, ex);
   }
-  if (!finite) {
-    L.cls = kNonFinite;
-    return L;
-  }
-  // Exact power-of-two pre-scale: the largest entry lands in [0.5, 1).  When
-  // every entry is zero or stays normal, by exponent arithmetic; otherwise
-  // (subnormal results or inputs, huge entries) by scalbn.
-  double a[6];
-  L.e = E - 1022;
+  if (!finite) return false;
+  e = E - 1022;
   bool exp_ok = (E >= 1 && E <= 2044);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     const int ex = (__double2hiint(a_in[i]) >> 20) & 0x7ff;
-    exp_ok &= is_zero(a_in[i]) || (ex >= 1 && ex - L.e >= 1);
+    exp_ok &= is_zero(a_in[i]) || (ex >= 1 && ex - e >= 1);
   }
   if (exp_ok) {
 #pragma unroll
     for (int i = 0; i < 6; ++i)
       a[i] = is_zero(a_in[i]) ? a_in[i]
-                              : __hiloint2double(__double2hiint(a_in[i]) - L.e * (1 << 20), __double2loint(a_in[i]));
+                              : __hiloint2double(__double2hiint(a_in[i]) - e * (1 << 20), __double2loint(a_in[i]));
   } else {
-    double amax = 0.0;
+    // The largest magnitude's exponent: of its bit pattern, or of its fraction
+    // when it is subnormal (0 for a zero matrix).
+    uint64_t top = 0;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) amax = fmax(amax, fabs(a_in[i]));
-    int e = 0;
-    if (amax > 0.0) frexp(amax, &e);
-    L.e = e;
+    for (int i = 0; i < 6; ++i) top = max(top, mag_bits(a_in[i]));
+    e = E > 0 ? E - 1022 : (top ? -1010 - __clzll((long long)top) : 0);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) a[i] = scalbn(a_in[i], -e);
+    for (int i = 0; i < 6; ++i) a[i] = scalbn_rare(a_in[i], -e);
+  }
+  return true;
+}
+
+// Phase A: pre-scale, Sec. 1 arrow reduction, Sec. 1.1 classification.
+// kEispack selects the EISPACK-style deflation test of Sec. 1.1 (the form
+// the paper starts from) instead of the simplified one it adopts.
+template <bool kEispack = false>
+__device__ __forceinline__ Lane make_lane(const double a_in[6]) {
+  Lane L;
+  double a[6];
+  if (!prescale(a_in, a, L.e)) {
+    L.cls = kNonFinite;
+    return L;
   }
   const Rot J = ordered_rotation(a[0], a[3], a[1]);
   L.a1 = J.l1;
@@ -416,7 +422,7 @@ __device__ __forceinline__ Lane make_lane(const double a_in[6]) {
                               : (kCDefl * kEps) * fabs(L.a1 + L.a2) * h2;
   if (dbits(h2) == 0)
     L.cls = kDiagonal;
-  else if (dbits(fabs(abar * b1 * b2)) <= dbits(rhs))
+  else if (mag_bits(abar * b1 * b2) <= dbits(rhs))
     L.cls = kDeflated;  // also the exact beta- and combo-deflations
   else
     L.cls = kReduced;

@@ -1,0 +1,426 @@
+// solve_fx.cuh -- FP64 eigenpairs from an FP32 solve, refined in 62-bit fixed
+// point on the integer pipes.
+//
+// GB300 executes 1.68 FP64 lanes per clock per SM but 64 lanes of the 32 x 32
+// -> 64 bit product and of a 64-bit addition (measured), so a fixed-point
+// multiply-add on 31-bit limbs (three products) costs a tenth of an FP64 one.
+// Packed doubles of similar size are held in fixed point with 62 fractional
+// bits, and absolute errors of 2^-60 are a hundredth of the FP64 rounding of
+// the eigenvalues.  A matrix whose entries are all within 2^20 of the largest
+// is solved so:
+//   1. the method of C. F. Borges (arXiv 1806.06698, Secs. 1-1.4.1) in FP32
+//      gives an approximate eigenvector frame, kept as a quaternion: R(q) is
+//      a rotation whatever the rounding of q, so no orthogonalisation follows;
+//   2. B = R^T A R in fixed point; the rotation that diagonalises it -- an
+//      exact Jacobi rotation (Golub and Van Loan, Matrix Computations, 8.5)
+//      of the closest pair, first-order perturbation towards the third -- is
+//      formed in FP32 and multiplied into q, now with 30-bit components;
+//   3. B is formed again from the new q.  Its off-diagonal entries are below
+//      2^-27 (checked), so its diagonal holds the eigenvalues, and first-order
+//      perturbation gives the eigenvectors: R (I + W + W^2/2), orthogonal to
+//      rounding, W_ij = B_ij/(B_jj - B_ii) (Kato, Perturbation Theory for
+//      Linear Operators, ch. 2).
+// A matrix that fails the entry or the off-diagonal check (graded or
+// structured entries, three close eigenvalues, FP32 roots that did not
+// converge) is left to the FP64 path.  The decision depends on the matrix
+// alone, never on its neighbours in the batch, and every FP32 sum of products
+// is an explicit fused operation, so that all builds of the kernels return
+// the same bits.
+#pragma once
+
+#include <cstdint>
+
+#include "arith.cuh"
+#include "solve_f32.cuh"
+
+namespace syev3 {
+namespace fx {
+namespace {  // internal linkage: every translation unit gets its own copy
+
+// Fixed-point scales, in fractional bits: matrix entries (of A/2 after the
+// pre-scale: |a/2| < 1/2) 62, rotation entries 60, A R and R^T A R 61.
+// A number is split into a signed upper and a non-negative lower limb,
+// v = h 2^31 + l (both with the sign of a for a matrix entry).  In a 3-term
+// sum of products the h h and the h l + l h parts accumulate in one 64-bit
+// register each; with the scales above neither overflows
+// (|sum h l + l h| < 2^31 (sum |h_a| + sum |h_b|) <= 3.9 x 2^61), and l l is
+// dropped, or replaced by its mean where that is not zero, through the
+// accumulator's start.
+struct Split {
+  int h, l;
+};
+
+__device__ __forceinline__ Split split31(const int64_t v) { return {(int)(v >> 31), (int)v & 0x7fffffff}; }
+
+// a b + c in one instruction (the plain expression was measured to become a
+// product and a separate 64-bit addition in places).
+__device__ __forceinline__ int64_t madw(const int a, const int b, const int64_t c) {
+  int64_t d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+__device__ __forceinline__ void dot3(const Split a0, const Split a1, const Split a2, const Split b0, const Split b1,
+                                     const Split b2, int64_t& hh, int64_t& cross) {
+  hh = madw(a2.h, b2.h, madw(a1.h, b1.h, (int64_t)a0.h * b0.h));
+  cross = madw(a0.h, b0.l, madw(a0.l, b0.h, cross));
+  cross = madw(a1.h, b1.l, madw(a1.l, b1.h, cross));
+  cross = madw(a2.h, b2.l, madw(a2.l, b2.h, cross));
+}
+
+// int64 -> float within 2^-23 relative: signed halves v = h 2^32 + l.
+__device__ __forceinline__ float to_float(const int64_t v) {
+  const int l = (int)v, h = (int)(v >> 32) + (int)((unsigned)l >> 31);
+  return fmaf((float)h, 0x1p32f, (float)l);
+}
+
+// v 2^-frac as a double, rounded once: the halves become exact doubles by
+// placing them in the fraction of a constant, so that two additions suffice.
+template <int kFrac>
+__device__ __forceinline__ double to_double(const int64_t v) {
+  // upper half: 2^a + x 2^(32-frac), x = upper word + 2^31; lower: 2^b + lo 2^-frac
+  constexpr int kHi = 1023 + 52 + 32 - kFrac, kLo = 1023 + 52 - kFrac;
+  const double dh = __hiloint2double(kHi << 20, (int)((unsigned)(v >> 32) ^ 0x80000000u));
+  const double dl = __hiloint2double(kLo << 20, (int)v);
+  constexpr double u = 1.0 / (double)(1ull << (kFrac - 32));  // 2^(32-frac)
+  constexpr double off = 0x1p52 * u + 0x1p31 * u + 0x1p20 * u;
+  return (dh - off) + dl;
+}
+
+// v 2^(e-frac) as a double on the integer pipes, |v| < 2^63: normalised, rounded
+// to nearest with ties away (v carries rounding errors of its own), the
+// exponent added.  A zero upper word of |v| takes the form above, a result
+// out of the normal range the general scaling; both rare.
+template <int kFrac>
+__device__ __forceinline__ double to_double_int(const int64_t v, const int e = 0) {
+  const int64_t s = v >> 63;
+  const uint64_t m = (uint64_t)((v ^ s) - s);
+  const unsigned hi = (unsigned)(m >> 32), lo = (unsigned)m;
+  if (hi == 0u) return mul_pow2(to_double<kFrac>(v), e);
+  const int z = __clz((int)hi);
+  const unsigned mh = __funnelshift_l(lo, hi, z), ml = lo << z;
+  const uint64_t f = (((uint64_t)mh << 32 | ml) >> 11) + ((ml >> 10) & 1u);  // 53 bits, rounded
+  const int E = 1023 + 62 - kFrac - z;  // exponent field at e = 0, less the leading bit's carry
+  const int sign = (int)(s << 31);
+  if ((unsigned)(E + e) > 2044u)
+    return mul_pow2(__hiloint2double(((int)(f >> 32) + (E << 20)) | sign, (int)f), e);
+  return __hiloint2double(((int)(f >> 32) + ((E + e) << 20)) | sign, (int)f);
+}
+
+// Rotation entries x 2^60 from an integer quaternion q with |q|^2 = 2^60
+// (1 + eta): the numerators of R(q), row by row; norm receives |q|^2.
+struct Quat {
+  int w, x, y, z;
+};
+
+__device__ __forceinline__ void rotation(const Quat q, int64_t R[9], int64_t& norm) {
+  const int64_t ww = (int64_t)q.w * q.w, xx = (int64_t)q.x * q.x, yy = (int64_t)q.y * q.y, zz = (int64_t)q.z * q.z;
+  const int64_t s = ww - zz, d = xx - yy, p = ww + zz, e = xx + yy;
+  norm = p + e;
+  R[0] = s + d;
+  R[4] = s - d;
+  R[8] = p - e;
+  const int64_t xy = (int64_t)q.x * q.y, xz = (int64_t)q.x * q.z, yz = (int64_t)q.y * q.z;
+  const int w2 = 2 * q.w;
+  R[1] = 2 * xy - (int64_t)w2 * q.z;
+  R[3] = madw(w2, q.z, 2 * xy);
+  R[2] = madw(w2, q.y, 2 * xz);
+  R[6] = 2 * xz - (int64_t)w2 * q.y;
+  R[5] = 2 * yz - (int64_t)w2 * q.x;
+  R[7] = madw(w2, q.x, 2 * yz);
+}
+
+// R^T (A/2) R x 2^61 (upper triangle 00 01 11 02 12 22); a holds the limbs of
+// the packed A/2 (11, 22, 33, 12, 13, 23) x 2^62.
+__device__ __forceinline__ void rotated(const Split a[6], const Split r[9], int64_t B[6]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    Split t[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const Split a0 = i == 0 ? a[0] : (i == 1 ? a[3] : a[4]);
+      const Split a1 = i == 0 ? a[3] : (i == 1 ? a[1] : a[5]);
+      const Split a2 = i == 0 ? a[4] : (i == 1 ? a[5] : a[2]);
+      int64_t hh, cross = 1ll << 29;  // half a unit (the l l terms' signs are those of a)
+      dot3(a0, a1, a2, r[j], r[3 + j], r[6 + j], hh, cross);
+      t[i] = split31((hh << 1) + (cross >> 30));
+    }
+#pragma unroll
+    for (int i = 0; i <= j; ++i) {
+      int64_t hh, cross = 0x70000000ll;  // mean of the l l terms (3 x 2^29) and half a unit
+      dot3(t[0], t[1], t[2], r[i], r[3 + i], r[6 + i], hh, cross);
+      B[j * (j + 1) / 2 + i] = (hh << 2) + (cross >> 29);
+    }
+  }
+}
+
+// The eigenvector frame of a (|a| < 1) by the FP32 method: outer
+// eigenvectors u1 and u3 by their closed forms (or the deflated 2x2 solve),
+// the third axis as their cross product; returned as an unnormalised
+// quaternion with |q| in [2, 4].
+struct QuatF {
+  float w, x, y, z;
+};
+
+__device__ __forceinline__ QuatF frame32(const float a[6]) {
+  using namespace f32;
+  const Rot32 J = ordered_rotation32(a[0], a[3], a[1]);
+  const float a1 = J.l1, a2 = J.l2, g = a[2];
+  const float b1 = fmaf(J.c, a[4], J.s * a[5]), b2 = fmaf(J.c, a[5], -J.s * a[4]);
+  const float ab = a1 - a2, bb1 = b1 * b1, bb2 = b2 * b2, h2 = fmaf(b1, b1, bb2);
+  float v[3], u[3];
+  if (fabsf(ab * b1 * b2) <= 0x1p-23f * fabsf(a1 + a2) * h2) {  // Sec. 1.1: deflated
+    const float rh = h2 > 0.f ? rsqrt32(h2) : 0.f, h = h2 * rh;
+    const float gs = b1 * rh, gc = h2 > 0.f ? b2 * rh : 1.f;
+    const Rot32 K = ordered_rotation32(fmaf(a1 * gs, gs, a2 * gc * gc), h, g);
+    v[0] = gc; v[1] = -gs; v[2] = 0.f;
+    u[0] = -gs * K.s; u[1] = -gc * K.s; u[2] = K.c;
+  } else {
+    float x[2];
+    bool more[2];
+    const P2 rab = pp(rcp32(ab)), b1p = make_float2(bb1, bb2), b2p = make_float2(bb2, bb1);
+    const P2 g2 = psub(make_float2(g, a2), make_float2(a1, g));
+    const P2 c = pmul(b2p, rab);
+    roots32x2(pp(ab), rab, b1p, b2p, g2, c, psub(make_float2(-g2.x, -g2.y), c), x, more);
+    const float mpa = x[0] + ab, npa = x[1] + ab;
+    v[0] = b1 * mpa; v[1] = b2 * x[0]; v[2] = x[0] * mpa;
+    u[0] = b1 * x[1]; u[1] = b2 * npa; u[2] = -(x[1] * npa);
+    const float iv = rsqrt32(fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2])));
+    const float iu = rsqrt32(fmaf(u[0], u[0], fmaf(u[1], u[1], u[2] * u[2])));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      v[i] *= iv;
+      u[i] *= iu;
+    }
+  }
+  // Columns v, u x v, u of the frame in the input's axes.
+  const float r00 = fmaf(J.c, v[0], -J.s * v[1]), r10 = fmaf(J.s, v[0], J.c * v[1]), r20 = v[2];
+  const float r02 = fmaf(J.c, u[0], -J.s * u[1]), r12 = fmaf(J.s, u[0], J.c * u[1]), r22 = u[2];
+  const float r01 = fmaf(r12, r20, -r22 * r10), r11 = fmaf(r22, r00, -r02 * r20), r21 = fmaf(r02, r10, -r12 * r00);
+  // 4 q_m q for the largest component q_m of the unit quaternion, read off
+  // the rotation matrix (Shepperd 1978).
+  const float ax = r21 - r12, ay = r02 - r20, az = r10 - r01, sxy = r01 + r10, sxz = r02 + r20, syz = r12 + r21;
+  const bool neg = r22 < 0.f, s = neg ? r00 > r11 : r00 < -r11;
+  const float d0 = neg ? 1.f - r22 : 1.f + r22, d1 = neg ? r00 - r11 : r00 + r11;
+  const float t = s == neg ? d0 + d1 : d0 - d1;  // x and w cases add, y and z subtract
+  QuatF q;
+  if (neg) {
+    q.w = s ? ax : ay;
+    q.x = s ? t : sxy;
+    q.y = s ? sxy : t;
+    q.z = s ? sxz : syz;
+  } else {
+    q.w = s ? az : t;
+    q.x = s ? sxz : ax;
+    q.y = s ? syz : ay;
+    q.z = s ? t : az;
+  }
+  return q;
+}
+
+// Step 2's rotation for B = (00 01 11 02 12 22): the closest pair (i, j) by a
+// Jacobi rotation about the third axis k with the couplings to k eliminated
+// to second order, then both towards k to first order; (i, j, k) cyclic.
+// Returns the vector part x 2^30 of the quaternion (1; p).  Only ratios of B
+// enter, so its scale is free.
+__device__ __forceinline__ void small_rotation(const int64_t B[6], int p[3]) {
+  const float e01 = to_float(B[1]), e02 = to_float(B[3]), e12 = to_float(B[4]);
+  const float g01 = to_float(B[2] - B[0]), g12 = to_float(B[5] - B[2]), g02 = to_float(B[5] - B[0]);
+  const float m01 = fabsf(g01), m12 = fabsf(g12), m02 = fabsf(g02);
+  const bool k2 = m01 <= m12 && m01 <= m02, k0 = !k2 && m12 <= m02;  // else k = 1
+  const float e = k2 ? e01 : (k0 ? e12 : e02), g = k2 ? g01 : (k0 ? g12 : -g02);
+  const float fi = k2 ? e02 : (k0 ? e01 : e12), fj = k2 ? e12 : (k0 ? e02 : e01);
+  const float ri = rcp32(k2 ? -g02 : (k0 ? g01 : g12)), rj = rcp32(k2 ? -g12 : (k0 ? g02 : -g01));
+  const float wi = fi * ri, wj = fj * rj;
+  const float ee = fmaf(0.5f, fmaf(fi, wj, fj * wi), e), gg = g + fmaf(fj, wj, -fi * wi);
+  const float den = fabsf(gg) + sqrt32(fmaf(gg, gg, 4.f * ee * ee));
+  float t = den > 0.f ? -2.f * ee * rcp32(den) : 0.f;
+  t = gg < 0.f ? -t : t;
+  const float h = t * rcp32(1.f + sqrt32(fmaf(t, t, 1.f)));  // tan of half the angle
+  const float r = rcp32(fmaf(h, h, 1.f)), c = fmaf(2.f, r, -1.f), s = 2.f * h * r;
+  const float oi = fmaf(c, fj, -s * fi) * rj, oj = -fmaf(c, fi, s * fj) * ri;
+  const int pi = __float2int_rn(0x1p29f * fmaf(-h, oj, oi)), pj = __float2int_rn(0x1p29f * fmaf(h, oi, oj));
+  const int pk = __float2int_rn(0x1p30f * h);
+  p[0] = k2 ? pi : (k0 ? pk : pj);
+  p[1] = k2 ? pj : (k0 ? pi : pk);
+  p[2] = k2 ? pk : (k0 ? pj : pi);
+}
+
+// q (1; p), the components x 2^30 (|p| <= 1: the result is below 2^31).
+__device__ __forceinline__ Quat times(const Quat q, const int p[3]) {
+  constexpr int64_t half = 1ll << 29;
+  Quat o;
+  o.w = q.w - (int)(madw(q.z, p[2], madw(q.y, p[1], madw(q.x, p[0], half))) >> 30);
+  o.x = q.x + (int)(madw(-q.z, p[1], madw(q.y, p[2], madw(q.w, p[0], half))) >> 30);
+  o.y = q.y + (int)(madw(-q.x, p[2], madw(q.z, p[0], madw(q.w, p[1], half))) >> 30);
+  o.z = q.z + (int)(madw(-q.y, p[0], madw(q.x, p[1], madw(q.w, p[2], half))) >> 30);
+  return o;
+}
+
+// q scaled to |q|^2 = 2^60 (1 + eta), |eta| < 2^-27: an FP32 inverse square
+// root with one Newton correction of the residual N s^2 - 1 (from 32-bit
+// limbs, to 2^-30).
+__device__ __forceinline__ Quat normalised(const Quat q) {
+  const int64_t N = madw(q.z, q.z, madw(q.y, q.y, madw(q.x, q.x, (int64_t)q.w * q.w)));  // [2^59, 2^61)
+  const int n31 = (int)(N >> 31);                     // N / 2^60 x 2^29
+  const float s = rsqrt32((float)n31 * 0x1p-29f);     // (1/2, sqrt 2]
+  const int si = __float2int_rn(s * 0x1p30f);         // exact
+  const int s2 = (int)(((int64_t)si * si) >> 31);     // s^2 x 2^29
+  const int res = (int)(((int64_t)n31 * s2 - (1ll << 58)) >> 27);  // (N s^2 - 1) x 2^31
+  const int sc = si - (int)(((int64_t)si * res) >> 32);            // s (1 - res/2) x 2^30
+  constexpr int64_t half = 1ll << 29;
+  Quat o;
+  o.w = (int)(madw(q.w, sc, half) >> 30);
+  o.x = (int)(madw(q.x, sc, half) >> 30);
+  o.y = (int)(madw(q.y, sc, half) >> 30);
+  o.z = (int)(madw(q.z, sc, half) >> 30);
+  return o;
+}
+
+// Largest off-diagonal entry of the second B, 2^-27 (x 2^61); the rounding of
+// q to 30 bits leaves up to 2^-28.
+constexpr float kOffMax = 0x1p34f;
+// Largest first-order rotation: W is held x 2^53 in 31 bits.
+constexpr float kRotMax = 0x1p-23f;
+// Largest second-order change of an eigenvalue, w e, 2^-56 (x 2^61): the same
+// bound keeps the vectors' second-order terms below 2^-56 over their gap.
+constexpr float kSecond = 0x1p5f;
+// Off-diagonal entries at the rounding level of B (up to 2^-56) between values
+// that are equal to that level: any vectors of the pair's plane will do.
+constexpr float kNoise = 0x1p5f;
+
+// e / g with the reciprocal's 2^-23 corrected by one Newton step.
+__device__ __forceinline__ float quotient(const float e, const float g) {
+  const float r = rcp32(g);
+  return e * fmaf(r, fmaf(-g, r, 1.f), r);
+}
+
+// The packed matrix A as limbs of A 2^-e/2, its largest entry in [1/4, 1/2),
+// when every off-diagonal entry is within 2^20 of the largest entry's exponent
+// and every diagonal one is so or zero (similar), or there is no off-diagonal
+// entry at all (diagonal); neither for a non-finite entry.  Entries within
+// 2^8 are held exactly, smaller ones to 2^-62; wider spreads are left to the
+// FP64 path, which keeps small entries to their own relative accuracy.
+constexpr unsigned kSpread = 20;
+
+struct Fixed {
+  Split a[6];
+  int e;
+  bool similar, diagonal, finite;
+};
+
+__device__ __forceinline__ Fixed fixed_of(const double a_in[6]) {
+  Fixed F;
+  unsigned h[6], l[6], top = 0u;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    h[i] = (unsigned)__double2hiint(a_in[i]);
+    l[i] = (unsigned)__double2loint(a_in[i]);
+    top = max(top, h[i] & 0x7fffffffu);
+  }
+  F.finite = top < 0x7ff00000u;
+  F.diagonal = (((h[3] | h[4] | h[5]) << 1) | l[3] | l[4] | l[5]) == 0u;
+  int shift = 0;
+  if (top < (64u << 20)) {  // subnormal entries may be near: scale up, exactly
+    shift = 256;
+    top = 0u;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const double x = scalbn_rare(a_in[i], shift);
+      h[i] = (unsigned)__double2hiint(x);
+      l[i] = (unsigned)__double2loint(x);
+      top = max(top, h[i] & 0x7fffffffu);
+    }
+  }
+  const int E = (int)(top >> 20);
+  F.e = E - 1022 - shift;
+  unsigned far = 0u;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int d = E - (int)((h[i] >> 20) & 0x7ffu);
+    const bool zero = i < 3 && ((h[i] << 1) | l[i]) == 0u;
+    far = max(far, zero ? 0u : (unsigned)d);
+    const int sign = zero ? 0 : (((int)h[i] >> 31) | 1);
+    const unsigned m = (h[i] & 0xfffffu) | 0x100000u;  // 53-bit fraction m : l
+    const unsigned y1 = __funnelshift_l(l[i], m, 8) >> (d & 31), y0 = __funnelshift_r(l[i] << 8, m << 8 | l[i] >> 24, d);
+    F.a[i].h = (int)__funnelshift_r(y0, y1, 31) * sign;
+    F.a[i].l = (int)(y0 & 0x7fffffffu) * sign;
+  }
+  F.similar = far <= kSpread;
+  return F;
+}
+
+// Eigenvalues l[3] and, with kVectors, eigenvectors U[i*3+k] of a matrix of
+// similar entries, without the sign rule; rk[k] is pair k's place in ascending order.
+// False when they could not be certified.
+template <bool kVectors>
+__device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], int rk[3]) {
+  const Split* const As = F.a;
+  float af[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) af[i] = (float)As[i].h * 0x1p-30f;
+  const QuatF f = frame32(af);
+  const float sc = 0x1p30f * rsqrt32(fmaf(f.w, f.w, fmaf(f.x, f.x, fmaf(f.y, f.y, f.z * f.z))));
+  Quat q = {__float2int_rn(f.w * sc), __float2int_rn(f.x * sc), __float2int_rn(f.y * sc), __float2int_rn(f.z * sc)};
+  int64_t R[9], N, B[6];
+  Split Rs[9];
+  rotation(q, R, N);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) Rs[i] = split31(R[i]);
+  rotated(As, Rs, B);
+  int p[3];
+  small_rotation(B, p);
+  q = normalised(times(q, p));
+  rotation(q, R, N);
+  const int eta = (int)((N - (1ll << 60)) >> 2);  // eta x 2^58
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    R[i] -= ((int64_t)(int)(R[i] >> 31) * eta) >> 27;
+    Rs[i] = split31(R[i]);
+  }
+  rotated(As, Rs, B);
+  float e01 = to_float(B[1]), e02 = to_float(B[3]), e12 = to_float(B[4]);
+  const float off = fmaxf(fabsf(e01), fmaxf(fabsf(e02), fabsf(e12)));
+  float w01 = quotient(e01, to_float(B[2] - B[0])), w02 = quotient(e02, to_float(B[5] - B[0])),
+        w12 = quotient(e12, to_float(B[5] - B[2]));
+  if (!(fabsf(w01) <= kRotMax) && fabsf(e01) <= kNoise) w01 = 0.f;
+  if (!(fabsf(w02) <= kRotMax) && fabsf(e02) <= kNoise) w02 = 0.f;
+  if (!(fabsf(w12) <= kRotMax) && fabsf(e12) <= kNoise) w12 = 0.f;
+  const float big = fmaxf(fabsf(w01), fmaxf(fabsf(w02), fabsf(w12)));
+  const float second = fmaxf(fabsf(w01 * e01), fmaxf(fabsf(w02 * e02), fabsf(w12 * e12)));
+  // (the last comparison fails for a NaN among the w, which the maxima drop)
+  if (!(off <= kOffMax && big <= kRotMax && second <= kSecond && w01 + w02 + w12 < 1.f)) return false;
+  // B is of A/2: at 2^60 its diagonal is the eigenvalues'.
+  rk[0] = (int)(B[2] < B[0]) + (int)(B[5] < B[0]);
+  rk[1] = (int)(B[0] <= B[2]) + (int)(B[5] < B[2]);
+  rk[2] = (int)(B[0] <= B[5]) + (int)(B[2] <= B[5]);
+  l[0] = to_double_int<60>(B[0], F.e);
+  l[1] = to_double_int<60>(B[2], F.e);
+  l[2] = to_double_int<60>(B[5], F.e);
+  if (kVectors) {
+    // R (I + W + W^2/2), W antisymmetric: orthogonal to third order.
+    const int x01 = __float2int_rn(w01 * 0x1p53f), x02 = __float2int_rn(w02 * 0x1p53f),
+              x12 = __float2int_rn(w12 * 0x1p53f);
+    const float s02 = w02 * w02, s12 = w12 * w12;
+    const int n0 = __float2int_rn(-0x1p52f * fmaf(w01, w01, s02)), n1 = __float2int_rn(-0x1p52f * fmaf(w01, w01, s12)),
+              n2 = __float2int_rn(-0x1p52f * fmaf(w02, w02, s12));
+    const int y01 = __float2int_rn(-0x1p52f * w02 * w12), y02 = __float2int_rn(0x1p52f * w01 * w12),
+              y12 = __float2int_rn(-0x1p52f * w01 * w02);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int r0 = Rs[3 * i].h, r1 = Rs[3 * i + 1].h, r2 = Rs[3 * i + 2].h;  // x 2^29
+      constexpr int64_t half = 1ll << 20;
+      const int64_t d0 = madw(r2, y02 - x02, madw(r1, y01 - x01, madw(r0, n0, half)));  // x 2^82
+      const int64_t d1 = madw(r2, y12 - x12, madw(r1, n1, madw(r0, y01 + x01, half)));
+      const int64_t d2 = madw(r2, n2, madw(r1, y12 + x12, madw(r0, y02 + x02, half)));
+      U[i * 3 + 0] = to_double_int<61>((R[3 * i] << 1) + (d0 >> 21));
+      U[i * 3 + 1] = to_double_int<61>((R[3 * i + 1] << 1) + (d1 >> 21));
+      U[i * 3 + 2] = to_double_int<61>((R[3 * i + 2] << 1) + (d2 >> 21));
+    }
+  }
+  return true;
+}
+
+}  // namespace
+}  // namespace fx
+}  // namespace syev3

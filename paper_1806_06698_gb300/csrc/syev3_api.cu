@@ -212,6 +212,7 @@ int syev3_device_flags(uint32_t* flags) {
   if (e != cudaSuccess) return cuda_fail(e);
   unsigned v = 0;
   e = syev3::take_flags_f64(&v);
+  if (e == cudaSuccess) e = syev3::take_flags_f64_study(&v);
   if (e == cudaSuccess) e = syev3::take_flags_f32(&v);
   if (e == cudaSuccess) e = syev3::take_flags_bwd(&v);
   if (e != cudaSuccess) return cuda_fail(e);
