@@ -51,11 +51,11 @@ _CSRC = os.path.join(ROOT, "paper_1806_06698_gb300", "csrc")
 _COMMON = ["arith.cuh", "common.cuh", "internal.h", "../build.py"]
 TRAFFIC_CASES = {
     # case: (kernel, sources, workload)
-    "f64": ("k_syev3_f64", ["syev3_f64.cu", "solve_f64.cuh"] + _COMMON, "mixed FP64"),
-    "f32": ("k_syev3_f32", ["syev3_f32.cu", "solve_f64.cuh"] + _COMMON, "mixed FP32, plain"),
-    "f32c": ("k_syev3_f32", ["syev3_f32.cu", "solve_f64.cuh"] + _COMMON, "mixed FP32, compensated"),
-    "f32ws": ("k_syev3_f32", ["syev3_f32.cu", "solve_f64.cuh", "syev3_api.cu"] + _COMMON,
-              "mixed FP32, compensated through syev3_batched_ws (FP32 kernel; the refinement kernel is k_refine_f32)"),
+    "f64": ("k_syev3_f64", ["syev3_f64.cu", "solve_f32.cuh", "solve_f64.cuh", "solve_fx.cuh"] + _COMMON, "mixed FP64"),
+    "f32": ("k_syev3_f32", ["syev3_f32.cu", "solve_f32.cuh", "solve_f64.cuh", "solve_fx.cuh"] + _COMMON, "mixed FP32, plain"),
+    "f32c": ("k_syev3_f32", ["syev3_f32.cu", "solve_f32.cuh", "solve_f64.cuh", "solve_fx.cuh"] + _COMMON, "mixed FP32, compensated"),
+    "f32ws": ("k_syev3_f32", ["syev3_f32.cu", "solve_f32.cuh", "solve_f64.cuh", "solve_fx.cuh", "syev3_api.cu"] + _COMMON,
+              "mixed FP32, compensated through syev3_batched_ws (FP32 kernel; the refinement kernel is k_refine_list)"),
     "bwd64": ("k_syev3_bwd", ["syev3_bwd.cu"] + _COMMON, "spectral FP64 backward"),
     "bwd32": ("k_syev3_bwd", ["syev3_bwd.cu"] + _COMMON, "spectral FP32 backward"),
 }
@@ -384,7 +384,7 @@ def _fp32_legs(args, dev, stream, barrier, A64_dev):
                 "dtype": "f32", "n": n,
                 "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                              "traffic": traffic_per_launch({"plain": "f32", "compensated": "f32ws"}.get(mode, "f32c"), n),
-                             "kernel": "k_syev3_f32" + (" + k_refine_f32" if work is not None else ""),
+                             "kernel": "k_syev3_f32" + (" + k_refine_list" if work is not None else ""),
                              "peak_source": "MEASURED_PEAKS hbm_gbs"},
                 "fp64_refined_fraction": ctr[2].item() / n if comp else 0.0,
                 "max_dlambda_vs_fp64_kernel_eps32": dl / 2.0 ** -23,

@@ -45,7 +45,7 @@ typedef struct CUstream_st* syev3_stream_t;
 typedef enum {
   SYEV3_F64 = 0,             /* binary64 in and out */
   SYEV3_F32 = 1,             /* binary32 in and out, plain FP32 arithmetic */
-  SYEV3_F32_COMPENSATED = 2  /* binary32 in and out; compensated FP32 with FP64 refinement of flagged lanes */
+  SYEV3_F32_COMPENSATED = 2  /* binary32 in and out; compensated FP32 with refinement of flagged lanes beyond FP32 */
 } syev3_dtype;
 
 typedef enum {
@@ -77,7 +77,7 @@ int syev3_last_cuda_error(void);
  * Returns SYEV3_EINVAL (NULL A or lambda, n < 0, bad dtype, misaligned or
  * overlapping buffers) or SYEV3_ECUDA (launch failure); SYEV3_OK otherwise.
  * syev3_batched allocates no device memory and uses none beyond its
- * arguments: the FP64 refinement of the compensated FP32 form works on a
+ * arguments: the refinement of the compensated FP32 form works on a
  * shared-memory list inside the kernel (syev3_batched_ws takes a scratch
  * workspace from the caller instead).
  */
@@ -88,7 +88,7 @@ int syev3_batched(const void* A_packed6, int64_t n, void* lambda, void* U, int d
  *   d_counters : device, 4 x uint64, or NULL.  When given, the kernels add
  *                [0] lanes whose zero finder hit the step cap,
  *                [1] lanes with a non-finite input entry,
- *                [2] lanes refined in FP64 (SYEV3_F32_COMPENSATED only),
+ *                [2] lanes refined (SYEV3_F32_COMPENSATED only),
  *                [3] refined lanes whose FP64 residual ||A u - lambda u||
  *                    exceeded 16 eps32 ||A||_F (SYEV3_F32_COMPENSATED only).
  *                The caller zeroes them; they accumulate across calls.
@@ -97,19 +97,11 @@ int syev3_batched_ex(const void* A_packed6, int64_t n, void* lambda, void* U, in
                      uint64_t* d_counters, syev3_stream_t stream);
 
 /* syev3_batched_ws -- syev3_batched_ex with a caller-provided device
- * workspace.  For SYEV3_F32_COMPENSATED the FP64 refinement of flagged lanes
- * (not in the paper: see SYEV3_F32_COMPENSATED) then runs as a second kernel
- * over a list of those lanes kept in the workspace, so the FP32 kernel holds
- * no FP64 code (fewer registers, more resident warps): the faster path when
- * few lanes are flagged (syev3_batched refines them in the FP32 kernel, in
- * whole warps gathered across tiles, and is the faster one when many are).
- * Results equal those of syev3_batched up to rounding.  From 2^21 matrices
- * on, the FP32 solve runs in 8 runs on `stream` and each run's refinement
- * on a side stream beside the next run's solve (events order them; `stream`
- * waits for the side stream before anything queued after the call); the
- * side stream and its events are created by the library on the first such
- * call for a device and kept, and calls from several host threads enqueue
- * their work one after the other.
+ * workspace.  For SYEV3_F32_COMPENSATED and 2^21 matrices or more the flagged
+ * matrices (not in the paper: see SYEV3_F32_COMPENSATED) are listed in the
+ * workspace and refined by a second kernel on `stream`, so that the FP32
+ * kernel needs fewer registers: the faster path for large batches.  Smaller
+ * ones take the path of syev3_batched.  Results equal those of syev3_batched.
  * Other dtypes ignore the workspace (it may be NULL).
  *   d_workspace     : device, at least syev3_workspace_bytes(n, dtype) bytes,
  *                     256-byte aligned, caller-owned; must not overlap the
@@ -125,26 +117,15 @@ size_t syev3_workspace_bytes(int64_t n, int dtype);
 int syev3_batched_ws(const void* A_packed6, int64_t n, void* lambda, void* U, int dtype, uint64_t* d_counters,
                      void* d_workspace, size_t workspace_bytes, syev3_stream_t stream);
 
-/* syev3_batched_static_ws -- syev3_batched_ws for SYEV3_F32_COMPENSATED
- * with the scratch list in the library's static device memory (a file-scope
- * __device__ array of SYEV3_STATIC_MAX_N records, 12.6 MB), so that the call
- * allocates nothing and needs no workspace from the caller.  Not in the
- * paper (which has no counterpart to any of the memory management here):
- * for callers that cannot pass a workspace -- a C caller without a device
- * allocator of its own, or code that must not call cudaMalloc/cudaFree on
- * this path (they synchronise the device and can fail under memory
- * pressure).
+/* syev3_batched_static_ws -- syev3_batched_ex with dtype
+ * SYEV3_F32_COMPENSATED for callers that must not allocate on this path: it
+ * takes no workspace and allocates nothing.
  *   A_packed6, lambda, U, d_counters, stream: as syev3_batched_ex with
  *   dtype SYEV3_F32_COMPENSATED (float32 buffers).
  *   n : 0 <= n <= SYEV3_STATIC_MAX_N, else SYEV3_EINVAL (nothing launched).
- * The array is shared by every call on a device: calls that overlap in time
- * (other streams or host threads) race on it and must be ordered by the
- * caller.  The first call on a device resolves the array's address
- * (cudaGetSymbolAddress, with that device current); it must come before any
- * stream capture begins on that device.  The address is kept for the life
- * of the process: do not use this entry point on a device after
- * cudaDeviceReset (the new context may place the array elsewhere).  Errors
- * as syev3_batched_ws. */
+ * (The limit is that of a scratch array the library no longer has; calls may
+ * overlap in time and may be the first on a device inside a stream capture.)
+ * Errors as syev3_batched_ex. */
 #define SYEV3_STATIC_MAX_N 262144
 
 int syev3_batched_static_ws(const void* A_packed6, int64_t n, void* lambda, void* U, uint64_t* d_counters,

@@ -84,4 +84,23 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// Shared -> global bulk copy, one bulk group per call; dst, src 16-byte
+// aligned, bytes a multiple of 16.  The caller makes the CTA's writes to src
+// visible to it first (fence_async_shared after a barrier of the writers) and
+// waits for the reads of src (bulk_read_wait) before src is written again or
+// the thread ends.
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// All bulk groups of this thread have finished reading shared memory.
+__device__ __forceinline__ void bulk_read_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
+// All bulk groups of this thread have also finished writing global memory.
+__device__ __forceinline__ void bulk_write_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 }  // namespace syev3

@@ -31,20 +31,12 @@ cudaError_t launch_f64_method(const double* A, int64_t n, double* lam, double* U
 cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool compensated,
                        unsigned long long* counters, cudaStream_t stream);
 
-// Compensated FP32 with the refinement deferred to a second kernel
-// (syev3_batched_ws): the workspace holds two counters at offset 0 and, from
-// kFlagListOffset, room for n records of flagged lanes: reduced arrows from
-// the front (counter 0), the other classes from the back (counter 1).
-struct alignas(16) FlagRec {
-  float v[9];       // a1 a2 b1 b2 g c s (pre-scaled arrow and rotation), mu, nu
-  int code;         // e << 2 | class
-  long long gidx;   // index of the matrix in the batch
-};
-static_assert(sizeof(FlagRec) == 48, "FlagRec layout");
+// Compensated FP32 with a workspace (syev3_batched_ws): a counter at offset 0
+// and, from kFlagListOffset, the rows of the flagged matrices.  (The header
+// grants 48 bytes per matrix; 8 are used.)
 constexpr size_t kFlagListOffset = 256;
-size_t f32c_workspace_bytes(int64_t n);
-cudaError_t launch_f32c_deferred(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters,
-                                 void* work, cudaStream_t stream);
+cudaError_t launch_f32c_ws(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters, void* work,
+                           cudaStream_t stream);
 
 // Serving: the work of one round, built on the device by the admission
 // kernel (serve.cu) and read by the solve kernels' serving instantiations.

@@ -421,6 +421,17 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   return true;
 }
 
+// Sign rule of column k of U: its largest-magnitude component, the first of
+// equals, becomes positive (magnitudes compared as integers, sign bits
+// flipped).
+__device__ __forceinline__ void sign_rule(double U[9], const int k) {
+  const uint64_t m0 = mag_bits(U[k]), m1 = mag_bits(U[3 + k]), m2 = mag_bits(U[6 + k]);
+  const double big = (m2 > m0 && m2 > m1) ? U[6 + k] : ((m1 > m0) ? U[3 + k] : U[k]);
+  const int flip = __double2hiint(big) & (int)0x80000000;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) U[i * 3 + k] = flip_sign(U[i * 3 + k], flip);
+}
+
 }  // namespace
 }  // namespace fx
 }  // namespace syev3

@@ -111,7 +111,7 @@ int syev3_batched(const void* A_packed6, int64_t n, void* lambda, void* U, int d
 
 size_t syev3_workspace_bytes(int64_t n, int dtype) {
   if (n <= 0 || dtype != SYEV3_F32_COMPENSATED) return 0;
-  return syev3::f32c_workspace_bytes(n);
+  return syev3::kFlagListOffset + (size_t)n * 48;
 }
 
 int syev3_batched_ws(const void* A_packed6, int64_t n, void* lambda, void* U, int dtype, uint64_t* d_counters,
@@ -121,17 +121,23 @@ int syev3_batched_ws(const void* A_packed6, int64_t n, void* lambda, void* U, in
   const int st = check_forward(A_packed6, n, lambda, U, dtype);
   if (st != SYEV3_OK || n == 0) return st;
   if (d_counters && (!aligned(d_counters, 8) || !device_accessible(d_counters))) return SYEV3_EINVAL;
-  const size_t need = syev3::f32c_workspace_bytes(n);
+  const size_t need = syev3_workspace_bytes(n, dtype);
   if (d_workspace == nullptr || workspace_bytes < need || !aligned(d_workspace, 256) ||
       !device_accessible(d_workspace))
     return SYEV3_EINVAL;
   if (overlap(d_workspace, need, A_packed6, (size_t)n * 24) || overlap(d_workspace, need, lambda, (size_t)n * 12) ||
       overlap(d_workspace, need, U, (size_t)n * 36))
     return SYEV3_EINVAL;
-  const cudaError_t e = syev3::launch_f32c_deferred(
+  const cudaError_t e = syev3::launch_f32c_ws(
       static_cast<const float*>(A_packed6), n, static_cast<float*>(lambda), static_cast<float*>(U),
       reinterpret_cast<unsigned long long*>(d_counters), d_workspace, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? SYEV3_OK : cuda_fail(e);
+}
+
+int syev3_batched_static_ws(const void* A_packed6, int64_t n, void* lambda, void* U, uint64_t* d_counters,
+                            syev3_stream_t stream) {
+  if (n > SYEV3_STATIC_MAX_N) return SYEV3_EINVAL;
+  return syev3_batched_ex(A_packed6, n, lambda, U, SYEV3_F32_COMPENSATED, d_counters, stream);
 }
 
 int syev3_batched_method(const void* A_packed6, int64_t n, void* lambda, void* U, int dtype,

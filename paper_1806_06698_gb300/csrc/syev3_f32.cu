@@ -14,17 +14,17 @@
 //    are clearly apart, with double-float (error-free transformation)
 //    products where they are close;
 //  * a double-float evaluation of the spectral function at the FP32 root
-//    and one Newton correction (Sec. 1.4.2) with it;
-// and uses FP64 only on the lanes it flags -- near-deflated (the test's two
-// sides within a factor kNearDefl), clustered (a relative eigenvalue gap
-// below kClusterTau) or capped -- for a final FP64 Newton step on mu and nu,
-// eigenvectors re-formed (and so re-orthogonalised) in FP64 and an FP64
-// residual check against the input.  Flagged lanes are compacted with warp
-// ballots into a shared-memory list and refined in whole warps, the rest
-// carried from tile to tile, so the FP64 work runs on as few warps as
-// possible; no global scratch memory is used (syev3_batched_ws instead
-// appends them to a list in a workspace for k_refine_f32, which runs beside
-// the FP32 solve on a second stream for large batches).
+//    and one Newton correction (Sec. 1.4.2) with it,
+// and refines the matrices it flags -- near-deflated (the test's two sides
+// within a factor kNearDefl), clustered (a relative eigenvalue gap below
+// kClusterTau) or capped -- from their input records: in 62-bit fixed point
+// (solve_fx.cuh), or, for graded or structured ones, by a final FP64 Newton
+// step on mu and nu and eigenvectors re-formed (and so re-orthogonalised) in
+// FP64; an FP64 residual check against the input feeds the counters.  A CTA
+// lists its flagged matrices in shared memory and refines them in whole warps
+// after its last tile; no global scratch memory is used (syev3_batched_ws
+// lists them in its workspace instead and refines them with a second kernel
+// for large batches).
 //
 // The two root problems of a lane (mu and nu) run the same expressions, so
 // their arithmetic is paired on the packed FP32 instructions (two correctly
@@ -34,20 +34,24 @@
 // __syncwarp over the lanes that form eigenpairs rejoins them for the common
 // tail (without it the warp was measured to stay split there).
 //
-// Memory path as in the FP64 kernel: tiles of kTPB records (24 B each) by
-// 1-D bulk copy into shared memory, double-buffered on mbarriers; results
-// staged in shared memory and written with 16-byte stores.  The plain form
-// moves 72 B per matrix; it is bound by instruction issue, not by HBM.
+// Memory path: tiles of kTPB records (24 B each) by 1-D bulk copy into shared
+// memory, double-buffered on mbarriers; a full tile's results leave their
+// staging rows by bulk copy too, so that no thread loads and stores them and
+// one barrier per tile fewer is needed (2^24 mixed matrices, plain: 415 us
+// against 484 with 16-byte stores by all threads).  The plain form moves 72 B
+// per matrix; it is bound by instruction issue (21.9 warp instructions per
+// matrix, 72 % of the slots), not by HBM.
 
 #include <cmath>
 #include <cstdint>
-#include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
 #include "serve_tile.cuh"
 #include "solve_f32.cuh"
 #include "solve_f64.cuh"
+#include "solve_fx.cuh"
 
 namespace syev3 {
 namespace {
@@ -72,7 +76,7 @@ constexpr float kTinySpike32 = 0x1p-60f;  // spikes below this are zeroed (beta-
 constexpr float kNearDefl = 2.0f;         // near-deflated: test sides within this factor
 constexpr float kClusterTau = 0x1p-23f;   // clustered: relative gap below this
 constexpr double kResidualTol = 16.0 * 0x1p-23;  // FP64 residual check, times ||A||_F
-constexpr int kPlain = 0, kInline = 1, kDeferred = 2;  // modes of k_syev3_f32
+constexpr int kPlain = 0, kComp32 = 1, kDeferred = 2;  // modes of k_syev3_f32
 
 constexpr int kDiag = f64::kDiagonal, kDefl = f64::kDeflated, kRed = f64::kReduced,
               kNonFin = f64::kNonFinite, kIdle = f64::kIdle;
@@ -190,28 +194,6 @@ __device__ __forceinline__ float bg_step32(const float ab, const float b1, const
   return (f > 0.f && xn < x) ? xn : x;
 }
 
-// The schedule of roots32x2 (below) one problem at a time, for the
-// compensated form with its refinement inside the kernel.  more[k] as in
-// roots32x2, for a move above 2^-12 x; the warp finishes such roots right
-// after.
-__device__ __forceinline__ void roots32(const float ab, const float b1[2], const float b2[2], const float g[2],
-                                        const float c[2], const float K[2], float x[2], bool more[2]) {
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    float f0, f1, x7;
-    bool model;
-    const float x0 = f64::start32(ab, b1[k], b2[k], g[k], c[k], K[k], x7, model);
-    float x1 = bg_step32(ab, b1[k], b2[k], g[k], c[k], K[k], x0, &f0);
-    const bool restart = model && !(f0 > 0.f);  // the small-root start was not right of the root
-    if (restart) x1 = x7;
-    const float x2 = bg_step32(ab, b1[k], b2[k], g[k], c[k], K[k], x1, &f1);
-    float f2;
-    const float x3 = bg_step32(ab, b1[k], b2[k], g[k], c[k], K[k], x2, &f2);
-    more[k] = (x2 - x3) > 0x1p-12f * x3;
-    x[k] = x3;
-  }
-}
-
 // Further steps for one problem until f/f' < C eps32 x (Sec. 1.4.1), f <= 0
 // or a stalled step; returns false if kMaxIt32 steps were not enough.  Not
 // inlined: it runs for few roots, and inlined it would weigh on the
@@ -277,59 +259,69 @@ __device__ __forceinline__ float newton_ff(const F2 ab, const F2 b1, const F2 b2
   return (xn > 0.f) ? xn : x;
 }
 
-// newton_ff for both problems at once (pairs as in roots32x2): each
-// double-float datum as a (head pair, low pair); ng = -g.  The same
-// expressions as newton_ff, term by term.
-__device__ __forceinline__ P2 pneg(const P2 a) { return pmul(a, pp(-1.f)); }
-
-__device__ __forceinline__ void ptwo_sum(const P2 a, const P2 b, P2& s, P2& e) {
-  s = padd(a, b);
-  const P2 bb = psub(s, a);
-  e = padd(psub(a, psub(s, bb)), psub(b, bb));
+// The roots (Sec. 1.2) of a lane: root[0] = mu, root[1] = nu (0 for the other
+// classes); with kComp, after one Newton correction in double-float.  Returns
+// whether the zero finder hit its step cap.  Every lane of the warp calls it.
+template <bool kComp>
+__device__ __forceinline__ bool roots_of(const Lane32& L, float root[2]) {
+  root[0] = root[1] = 0.f;
+  bool capped = false;
+  bool more[2] = {false, false};
+  float ab = 0.f, pb1[2] = {0.f, 0.f}, pb2[2] = {0.f, 0.f}, pg[2] = {0.f, 0.f};
+  if (L.cls == kRed) {
+    ab = L.a1 - L.a2;
+    roots_setup32(L, ab, pb1, pb2, pg);
+    const P2 rab = pp(rcp32(ab)), b1p = make_float2(pb1[0], pb1[1]), b2p = make_float2(pb2[0], pb2[1]);
+    const P2 g2 = make_float2(pg[0], pg[1]);
+    const P2 pc = pmul(b2p, rab);
+    roots32x2(pp(ab), rab, b1p, b2p, g2, pc, psub(make_float2(-g2.x, -g2.y), pc), root, more);
+  }
+  // Rare: roots still moving after the straight-line steps, finished in
+  // their own lanes (the warp runs this only when one of its roots needs it).
+  if (__any_sync(0xffffffffu, more[0] || more[1])) {
+    float xa = root[0], xb = root[1];
+    bool ca = false, cb = false;
+    if (more[0]) ca = !roots32_more(ab, pb1[0], pb2[0], pg[0], &xa);
+    if (more[1]) cb = !roots32_more(ab, pb1[1], pb2[1], pg[1], &xb);
+    root[0] = xa;
+    root[1] = xb;
+    capped = ca || cb;
+  }
+  if (kComp && L.cls == kRed) {
+    // Exact FP32 data as double-float, then one Newton correction with a
+    // double-float f at each root.
+    const F2 abf = two_sum(L.a1, -L.a2);
+    const float rabh = rcp32(abf.h);
+    const F2 fb1 = two_prod(L.b1, L.b1), fb2 = two_prod(L.b2, L.b2);
+    const F2 fg0 = two_sum(L.g, -L.a1), fg1 = two_sum(L.a2, -L.g);
+    // c = b2 / abar and K = -(g + c) as unnormalised pairs.
+    auto div_pair = [rabh, abf](const F2 num) {
+      const float q = num.h * rabh;
+      return F2{q, ((fmaf(-q, abf.h, num.h) + num.l) - q * abf.l) * rabh};
+    };
+    auto neg_sum_pair = [](const F2 a, const F2 b) {
+      const F2 t = two_sum(a.h, b.h);
+      return F2{-t.h, -((t.l + a.l) + b.l)};
+    };
+    const F2 fc0 = div_pair(fb2), fc1 = div_pair(fb1);
+    const F2 fK0 = neg_sum_pair(fg0, fc0), fK1 = neg_sum_pair(fg1, fc1);
+    root[0] = newton_ff(abf, fb1, fb2, fg0, fc0, fK0, root[0]);
+    root[1] = newton_ff(abf, fb2, fb1, fg1, fc1, fK1, root[1]);
+  }
+  return capped;
 }
 
-__device__ __forceinline__ P2 newton_ff2(const P2 abh, const P2 abl, const P2 b1h, const P2 b1l, const P2 b2h,
-                                        const P2 b2l, const P2 ngh, const P2 ngl, const P2 ch, const P2 cl,
-                                        const P2 Kh, const P2 Kl, const P2 x) {
-  const P2 r1 = prcp(x), nx = pneg(x);
-  P2 sh, s0l;
-  ptwo_sum(x, abh, sh, s0l);
-  const P2 sl = padd(s0l, abl);  // x + ab = sh + sl
-  const P2 r2 = prcp(sh);
-  // b1 / x: the quotient's head and the remainder over x.
-  const P2 q1 = pmul(b1h, r1);
-  const P2 q1l = pmul(padd(pfma(q1, nx, b1h), b1l), r1);
-  // Last term: + c x / (x + ab) below ab (the cancellation-free form),
-  // - b2 / (x + ab) above; numerator (nh, nl), quotient (q2, q2l).
-  const bool sx = x.x < abh.x, sy = x.y < abh.y;
-  const P2 cx = pmul(ch, x);
-  const P2 nh = psel(sx, sy, cx, b2h);
-  const P2 nl = psel(sx, sy, pfma(cl, x, pfma(ch, x, pneg(cx))), b2l);
-  const P2 q2 = pmul(nh, r2), nq2 = pneg(q2);
-  const P2 q2l = pmul(pfma(nq2, sl, padd(pfma(nq2, sh, nh), nl)), r2);
-  const P2 sg = psel(sx, sy, pp(1.f), pp(-1.f));
-  const P2 th = pmul(q2, sg), tl = pmul(q2l, sg);
-  const P2 lh = psel(sx, sy, Kh, ngh), ll = psel(sx, sy, Kl, ngl);
-  // Sum2 over x + lead - b1/x + last.
-  P2 uh, ul, vh, vl, wh, wl;
-  ptwo_sum(x, lh, uh, ul);
-  vh = psub(uh, q1);  // TwoSum(u.h, -q1)
-  {
-    const P2 bb = psub(vh, uh);
-    vl = psub(psub(uh, psub(vh, bb)), padd(q1, bb));
-  }
-  ptwo_sum(vh, th, wh, wl);
-  const P2 f = padd(wh, padd(padd(padd(ul, vl), padd(wl, ll)), psub(tl, q1l)));
-  const P2 fp = pfma(pmul(b2h, r2), r2, pfma(q1, r1, pp(1.f)));
-  const P2 xn = pfma(pneg(f), prcp(fp), x);
-  return psel(xn.x > 0.f, xn.y > 0.f, xn, x);
+// The sign bit of the largest-magnitude component, the first of equals.
+__device__ __forceinline__ unsigned sign_of_largest(const float y0, const float y1, const float y2) {
+  float big = (fabsf(y1) > fabsf(y0)) ? y1 : y0;
+  big = (fabsf(y2) > fabsf(big)) ? y2 : big;
+  return __float_as_uint(big) & 0x80000000u;
 }
 
 // Eigenpairs of a classified lane in FP32 (scaled frame); returns eigenvalues
 // ascending in l[] and vectors as columns in U[i*3+k].
 // Eigenvalues only: those of finish32 (the same expressions, compare order
 // and tie rule), ascending, in the scaled frame.
-template <bool kSync>
 __device__ __forceinline__ void finish32_values(const Lane32& L, float mu, float nu, float l_out[3],
                                                 const unsigned sync_mask) {
   const float a1 = L.a1, a2 = L.a2, b1 = L.b1, b2 = L.b2, g = L.g;
@@ -348,7 +340,7 @@ __device__ __forceinline__ void finish32_values(const Lane32& L, float mu, float
     l1 = (nu - mu) + g;
     l2 = a2 - nu;
   }
-  if constexpr (kSync) __syncwarp(sync_mask);  // the classes' lanes rejoin
+  __syncwarp(sync_mask);  // the classes' lanes rejoin
   float t;
   if (l1 < l0) { t = l0; l0 = l1; l1 = t; }
   if (l2 < l1) { t = l1; l1 = l2; l2 = t; }
@@ -356,7 +348,6 @@ __device__ __forceinline__ void finish32_values(const Lane32& L, float mu, float
   l_out[0] = l0; l_out[1] = l1; l_out[2] = l2;
 }
 
-template <bool kSync>
 __device__ __forceinline__ void finish32(const Lane32& L, float mu, float nu, float l_out[3], float U[9], int rk[3],
                                          const unsigned sync_mask) {
   const float a1 = L.a1, a2 = L.a2, b1 = L.b1, b2 = L.b2, g = L.g;
@@ -402,7 +393,7 @@ __device__ __forceinline__ void finish32(const Lane32& L, float mu, float nu, fl
       v[k][0] *= inv; v[k][1] *= inv; v[k][2] *= inv;
     }
   }
-  if constexpr (kSync) __syncwarp(sync_mask);  // the three classes' lanes rejoin for the common tail
+  __syncwarp(sync_mask);  // the three classes' lanes rejoin for the common tail
   float x[3][3];
 #pragma unroll
   for (int k = 0; k < 3; k += 2) {
@@ -434,9 +425,7 @@ __device__ __forceinline__ void finish32(const Lane32& L, float mu, float nu, fl
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const float y0 = x[k][0], y1 = x[k][1], y2 = x[k][2];
-    float big = (fabsf(y1) > fabsf(y0)) ? y1 : y0;
-    big = (fabsf(y2) > fabsf(big)) ? y2 : big;
-    const unsigned sb = __float_as_uint(big) & 0x80000000u;
+    const unsigned sb = sign_of_largest(y0, y1, y2);
     l_out[k] = l[k];
     U[0 * 3 + k] = __uint_as_float(__float_as_uint(y0) ^ sb);
     U[1 * 3 + k] = __uint_as_float(__float_as_uint(y1) ^ sb);
@@ -455,6 +444,28 @@ __device__ __forceinline__ void unscale3(float l[3], int e) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) l[k] = scalbnf(l[k], e);
   }
+}
+
+// The FP64 residual check ||A u - lambda u|| <= 16 eps32 ||A||_F of a refined
+// lane against its input record; true when it fails.
+__device__ __forceinline__ bool residual_fails(const float rec[6], const double lam[3], const double U[9]) {
+  const double M[3][3] = {{rec[0], rec[3], rec[4]}, {rec[3], rec[1], rec[5]}, {rec[4], rec[5], rec[2]}};
+  double nA = 0.0, worst = 0.0;
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) nA = fma(M[r][q], M[r][q], nA);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    double rr = 0.0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const double v = fma(M[r][0], U[k], fma(M[r][1], U[3 + k], fma(M[r][2], U[6 + k], -lam[k] * U[r * 3 + k])));
+      rr = fma(v, v, rr);
+    }
+    worst = fmax(worst, rr);
+  }
+  return !(worst <= kResidualTol * kResidualTol * nA);
 }
 
 // FP64 refinement of one flagged lane (compensated form): the arrow and the
@@ -478,70 +489,104 @@ __device__ __forceinline__ bool refine_one(const float f[9], const int code, con
     if (nu > 0.0) nu = f64::newton64(ab, bb2, bb1, g1, c1, -g1 - c1, nu);
   }
   f64::finish_lane(D, mu, nu, lam, U);
-  if (rec == nullptr) return false;
-  const double M[3][3] = {{rec[0], rec[3], rec[4]}, {rec[3], rec[1], rec[5]}, {rec[4], rec[5], rec[2]}};
-  double nA = 0.0, worst = 0.0;
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) nA = fma(M[r][q], M[r][q], nA);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double rr = 0.0;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const double v = fma(M[r][0], U[k], fma(M[r][1], U[3 + k], fma(M[r][2], U[6 + k], -lam[k] * U[r * 3 + k])));
-      rr = fma(v, v, rr);
-    }
-    worst = fmax(worst, rr);
-  }
-  return !(worst <= kResidualTol * kResidualTol * nA);
+  return rec != nullptr && residual_fails(rec, lam, U);
 }
 
-// kMode: kPlain (SYEV3_F32), kInline (compensated, flagged lanes refined in
-// FP64 inside the kernel on a shared-memory list) or kDeferred (compensated,
-// flagged lanes appended to a list in global memory -- the workspace of
-// syev3_batched_ws -- and refined by k_refine_f32; the kernel then holds no
-// FP64 code and needs fewer registers).
+// The refinement of one flagged matrix from its input record: in 62-bit fixed
+// point (solve_fx.cuh; about 2600 issue slots a warp, the FP64 pipe needs 8600
+// cycles) when its entries are of similar size, else refine_one on its FP32
+// arrow and roots, formed again by the FP32 solve's own steps.  out:
+// eigenvalues, then eigenvectors.  Whole warps call it; a lane without work
+// passes active = false.  Not inlined: all kernels then share its code and
+// return the same bits.
+__device__ __noinline__ bool refine_record(const float* rec, const bool active, const bool check, float out[12]) {
+  double lam[3], U[9];
+  int rk[3] = {0, 1, 2};
+  bool done = false, bad = false;
+  if (active) {
+    double a[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k] = f2d_exact(rec[k]);
+    const fx::Fixed F = fx::fixed_of(a);
+    if (F.similar && !F.diagonal && fx::solve<true>(F, lam, U, rk)) {
+      done = true;
+      bad = check && residual_fails(rec, lam, U);
+    }
+  }
+  if (__any_sync(0xffffffffu, active && !done)) {
+    Lane32 L;
+    L.cls = kIdle;
+    if (active && !done) L = make_lane32<true>(rec);
+    float root[2];
+    roots_of<true>(L, root);
+    if (active && !done) {
+      const float f[9] = {L.a1, L.a2, L.b1, L.b2, L.g, L.c, L.s, root[0], root[1]};
+      bad = refine_one(f, (L.e << 2) | L.cls, check ? rec : nullptr, lam, U);
+      rk[0] = 0; rk[1] = 1; rk[2] = 2;
+    }
+  }
+  if (active) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      out[rk[k]] = d2f_rn(lam[k]);
+      // The sign rule holds for the rounded components (two may become equal).
+      const float y0 = d2f_rn(U[k]), y1 = d2f_rn(U[3 + k]), y2 = d2f_rn(U[6 + k]);
+      const unsigned sb = sign_of_largest(y0, y1, y2);
+      out[3 + rk[k]] = __uint_as_float(__float_as_uint(y0) ^ sb);
+      out[6 + rk[k]] = __uint_as_float(__float_as_uint(y1) ^ sb);
+      out[9 + rk[k]] = __uint_as_float(__float_as_uint(y2) ^ sb);
+    }
+  }
+  return bad;
+}
+
+// Rows of a CTA's flagged matrices, refined after its last tile (or when a
+// further tile might not fit).
+template <bool kServe>
+struct FlagList;
+template <>
+struct FlagList<false> {
+  static constexpr int kCap = 1024;
+  uint32_t seq[kCap];  // place in the CTA's sequence of tiles x tile size + row
+};
+template <>
+struct FlagList<true> {
+  static constexpr int kCap = 512;
+  TileRef<float> at[kCap];  // the row's record and outputs
+};
+
+// kMode: kPlain (SYEV3_F32), kComp32 (compensated: the flagged matrices are
+// listed, and refined by the CTA's whole warps at the end) or kDeferred
+// (compensated: they are appended to a list in the caller's workspace, for
+// k_refine_list).  Refining at the end, the SM's warps run in step, which
+// matters for 40 KB of straight-line code: with 4 % of 2^22 matrices flagged
+// kComp32 takes 219 us; refined by single warps as soon as 32 had gathered,
+// 295; by FP64 code on a list per tile (the earlier form) 281.
 // kVectors = false (plain mode only): eigenvalues only, U_out NULL.
-// kServe: the serving build (plain or in-kernel compensated).  The tiles are
-// those of the device-resident work list `list` (A, n, lam_out and U_out are
-// unused), each with its own input and output rows; a tile's input is
-// bulk-copied from its first 16-byte boundary-aligned record on, or loaded
-// with plain loads when its start is not 16-byte aligned.  The production
-// builds (kServe = false) compile this out.
+// kServe: the serving build.  The tiles are those of the
+// device-resident work list `list` (A, n, lam_out and U_out are unused), each
+// with its own input and output rows; a tile's input is bulk-copied from its
+// first 16-byte boundary-aligned record on, or loaded with plain loads when
+// its start is not 16-byte aligned.  The production builds (kServe = false)
+// compile this out.
 template <bool kBulkIn, int kMode, bool kVectors = true, bool kServe = false>
-__global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A, int64_t n,
-                                                    float* __restrict__ lam_out, float* __restrict__ U_out,
-                                                    unsigned long long* __restrict__ counters,
-                                                    FlagRec* __restrict__ flag_list,
-                                                    unsigned long long* __restrict__ flag_count,
-                                                    const ServeList* __restrict__ list) {
+__global__ void __launch_bounds__(kTPB, kMode == kComp32 ? 6 : 1)
+    k_syev3_f32(const float* __restrict__ A, int64_t n, float* __restrict__ lam_out, float* __restrict__ U_out,
+                unsigned long long* __restrict__ counters, int64_t* __restrict__ flag_list,
+                unsigned long long* __restrict__ flag_count, const ServeList* __restrict__ list) {
   static_assert(!kServe || (kBulkIn && kMode != kDeferred && kVectors), "the serving build is bulk, vectors");
   static_assert(kTPB == kServeTile, "serving tiles are solve tiles");
-  constexpr bool kComp = kMode != kPlain;
-  constexpr bool kDefer = kMode == kDeferred;
+  constexpr bool kComp = kMode != kPlain, kList = kMode == kComp32;
   __shared__ alignas(16) float s_in[2][kTPB * 6];
   __shared__ alignas(16) float s_lam[kTPB * 3];
   __shared__ alignas(16) float s_U[kTPB * 9];
-  // Compensated form, refinement in the kernel: the list of flagged lanes,
-  // kFA floats each (arrow, roots, then the input record for the residual
-  // check), their codes and global indices.  Slots [0, nfc) hold the lanes
-  // carried from earlier tiles (fewer than 32), then this tile's.
-  constexpr int kFA = 15, kFW = kTPB + 32;
-  constexpr bool kInl = kMode == kInline;
-  __shared__ float s_fa[kInl ? kFA * kFW : 1];
-  __shared__ int s_fc[kInl ? kFW : 1];
-  __shared__ int64_t s_fg[kInl ? kFW : 1];
-  __shared__ int s_nflag;
   __shared__ alignas(8) uint64_t s_bar[2];
-  // Serving build: the tile of each buffer; the eigenvector row of each
-  // flagged lane in the list (s_fg then holds its eigenvalue row's address).
-  __shared__ TileRef<float> s_ref[kServe ? 2 : 1];
-  __shared__ float* s_fU[(kServe && kInl) ? kFW : 1];
+  __shared__ TileRef<float> s_ref[kServe ? 2 : 1];  // serving build: the tile of each buffer
+  constexpr int kCap = FlagList<kServe>::kCap;
+  __shared__ std::conditional_t<kList, FlagList<kServe>, int> s_list;
+  __shared__ int s_nflag;
 
   const int tid = threadIdx.x, lane_id = tid & 31;
-  const unsigned lt_mask = (1u << lane_id) - 1u;
   const int64_t n_tiles = kServe ? list->n_tiles : (n + kTPB - 1) / kTPB;
   bool want_U = (U_out != nullptr);
   bool vec_lam = ((reinterpret_cast<uintptr_t>(lam_out) & 15) == 0);
@@ -581,16 +626,62 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
     if (bytes) bulk_g2s(s_in[buf], A + base * 6, bytes, &s_bar[buf]);
   };
 
+  // Refines the listed matrices; every thread of the CTA calls it.
+  auto refine = [&]() {
+    if (tid == 0) bulk_write_wait();  // the FP32 results are in memory
+    __syncthreads();
+    const int count = s_nflag;
+    if constexpr (kList) {
+      for (int i0 = tid & ~31; i0 < count; i0 += kTPB) {  // whole warps
+        const bool active = i0 + lane_id < count;
+        float rec[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, out[12];
+        float *dl = nullptr, *dU = nullptr;
+        if (active) {
+          const float* src;
+          if constexpr (kServe) {
+            const TileRef<float> r = s_list.at[i0 + lane_id];
+            src = r.src;
+            dl = r.lam;
+            dU = r.U;
+          } else {
+            const uint32_t q = s_list.seq[i0 + lane_id];
+            const int64_t row = ((int64_t)(q / kTPB) * gridDim.x + blockIdx.x) * kTPB + q % kTPB;
+            src = A + row * 6;
+            dl = lam_out + row * 3;
+            dU = U_out ? U_out + row * 9 : nullptr;
+          }
+#pragma unroll
+          for (int k = 0; k < 6; ++k) rec[k] = src[k];
+        }
+        const bool bad = refine_record(rec, active, counters != nullptr, out);
+        if (bad) atomicAdd(&counters[3], 1ull);
+        if (active) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) dl[k] = out[k];
+          if (dU != nullptr) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) dU[k] = out[3 + k];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (tid == 0) s_nflag = 0;
+  };
+
   uint32_t phases = 0u;
-  int nfc = 0;  // flagged lanes carried into this tile (CTA-uniform)
+  uint32_t seq = (uint32_t)tid;  // this thread's row in the CTA's sequence of tiles
   int buf = 0;
   int64_t tile = blockIdx.x;
   if (kBulkIn && tid == 0 && tile < n_tiles) issue(tile, 0);
 
-  for (; tile < n_tiles; tile += gridDim.x, buf ^= 1) {
+  for (; tile < n_tiles; tile += gridDim.x, buf ^= 1, seq += kTPB) {
     const int64_t base = tile * kTPB;
     int cnt = (int)((n - base) < kTPB ? (n - base) : kTPB);
+    float* lam_tile = lam_out + base * 3;
+    float* U_tile = want_U ? U_out + base * 9 : nullptr;
     const int64_t next = tile + gridDim.x;
+    if (tid == 0) bulk_read_wait();  // the last tile's rows have left the staging area
     if (kBulkIn) {
       if (tid == 0 && next < n_tiles) issue(next, buf ^ 1);
       const bool ok = mbar_wait(&s_bar[buf], (phases >> buf) & 1u);
@@ -601,22 +692,25 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
         return;
       }
       phases ^= 1u << buf;
+      const float* src = A + base * 6;
+      int done_f = (int)((((uint32_t)cnt * 24u) & ~15u) / 4u);
       if constexpr (kServe) {
         const TileRef<float> r = s_ref[buf];
         cnt = r.cnt;
+        src = r.src;
+        lam_tile = r.lam;
+        U_tile = r.U;
         want_U = (r.U != nullptr);
         vec_lam = ((reinterpret_cast<uintptr_t>(r.lam) & 15) == 0);
         vec_U = want_U && ((reinterpret_cast<uintptr_t>(r.U) & 15) == 0);
-        const int done_f =
-            (reinterpret_cast<uintptr_t>(r.src) & 15) ? 0 : (int)((((uint32_t)cnt * 24u) & ~15u) / 4u);
-        for (int i = done_f + tid; i < cnt * 6; i += kTPB) s_in[buf][i] = r.src[i];
-        if (done_f < cnt * 6) __syncthreads();
-      } else {
-        const int done_f = (int)((((uint32_t)cnt * 24u) & ~15u) / 4u);
-        for (int i = done_f + tid; i < cnt * 6; i += kTPB) s_in[buf][i] = A[base * 6 + i];
-        if (done_f < cnt * 6) __syncthreads();
+        done_f = (reinterpret_cast<uintptr_t>(r.src) & 15) ? 0 : (int)((((uint32_t)cnt * 24u) & ~15u) / 4u);
+      }
+      if (done_f < cnt * 6) {
+        for (int i = done_f + tid; i < cnt * 6; i += kTPB) s_in[buf][i] = src[i];
+        __syncthreads();
       }
     } else {
+      __syncthreads();  // the previous tile's records and staging have been read
       for (int i = tid; i < cnt * 6; i += kTPB) s_in[buf][i] = A[base * 6 + i];
       __syncthreads();
     }
@@ -624,99 +718,17 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
     Lane32 L;
     L.cls = kIdle;
     L.near_defl = false;
-    float a_in[6];
     if (tid < cnt) {
       const float2* src = reinterpret_cast<const float2*>(&s_in[buf][tid * 6]);
       const float2 p0 = src[0], p1 = src[1], p2 = src[2];
-      a_in[0] = p0.x; a_in[1] = p0.y; a_in[2] = p1.x; a_in[3] = p1.y; a_in[4] = p2.x; a_in[5] = p2.y;
+      const float a_in[6] = {p0.x, p0.y, p1.x, p1.y, p2.x, p2.y};
       L = make_lane32<kComp>(a_in);
     }
-    // Plain and workspace forms: the warp's lanes that form eigenpairs (taken
-    // where all 32 are together), which rejoin after the class-specific part
-    // of the solve.
-    unsigned fin_mask = 0u;
-    if constexpr (kMode != kInline) fin_mask = __ballot_sync(0xffffffffu, L.cls != kIdle && L.cls != kNonFin);
-
-    // Roots (Sec. 1.2): problem 0 is mu, problem 1 is nu (spikes swapped).
-    float root[2] = {0.f, 0.f};
-    bool capped = false;
-    bool more[2] = {false, false};
-    float ab = 0.f, pb1[2] = {0.f, 0.f}, pb2[2] = {0.f, 0.f}, pg[2] = {0.f, 0.f};
-    if (L.cls == kRed) {
-      ab = L.a1 - L.a2;
-      if constexpr (kMode != kInline) {
-        roots_setup32(L, ab, pb1, pb2, pg);
-        const P2 rab = pp(rcp32(ab)), b1p = make_float2(pb1[0], pb1[1]), b2p = make_float2(pb2[0], pb2[1]);
-        const P2 g2 = make_float2(pg[0], pg[1]);
-        const P2 pc = pmul(b2p, rab);
-        roots32x2(pp(ab), rab, b1p, b2p, g2, pc, psub(make_float2(-g2.x, -g2.y), pc), root, more);
-      } else {
-        const float bb1 = L.b1 * L.b1, bb2 = L.b2 * L.b2;
-        pb1[0] = bb1; pb1[1] = bb2; pb2[0] = bb2; pb2[1] = bb1;
-        pg[0] = L.g - L.a1; pg[1] = L.a2 - L.g;
-        const float rab = rcp32(ab);
-        const float pc[2] = {pb2[0] * rab, pb2[1] * rab};
-        const float pK[2] = {-pg[0] - pc[0], -pg[1] - pc[1]};
-        roots32(ab, pb1, pb2, pg, pc, pK, root, more);
-      }
-    }
-    // Rare: roots still moving after the straight-line steps, finished in
-    // their own lanes (the warp runs this only when one of its roots needs it).
-    if (__any_sync(0xffffffffu, more[0] || more[1])) {
-      float xa = root[0], xb = root[1];
-      bool ca = false, cb = false;
-      if (more[0]) ca = !roots32_more(ab, pb1[0], pb2[0], pg[0], &xa);
-      if (more[1]) cb = !roots32_more(ab, pb1[1], pb2[1], pg[1], &xb);
-      root[0] = xa;
-      root[1] = xb;
-      capped = capped || ca || cb;
-    }
-    if (L.cls == kRed) {
-      if (kComp) {
-        if constexpr (kMode == kInline) {
-          // Exact FP32 data as double-float, then one Newton correction with
-          // a double-float f at each root (both problems paired; the
-          // workspace form keeps the scalar code: its 47 registers leave room
-          // for the refinement CTAs beside it).
-          const F2 abf = two_sum(L.a1, -L.a2);
-          const P2 abh = pp(abf.h), abl = pp(abf.l), rabh = pp(rcp32(abf.h));
-          // spikes (b1^2, b2^2) exactly; problem 1 has them swapped
-          const P2 B = make_float2(L.b1, L.b2);
-          const P2 bh = pmul(B, B), bl = pfma(B, B, pneg(bh));
-          const P2 sbh = make_float2(bh.y, bh.x), sbl = make_float2(bl.y, bl.x);
-          P2 gh, gl;  // (g - a1, a2 - g) exactly
-          ptwo_sum(make_float2(L.g, L.a2), make_float2(-L.a1, -L.g), gh, gl);
-          // c = b2 / abar and K = -(g + c) as unnormalised pairs.
-          const P2 ch = pmul(sbh, rabh);
-          const P2 cl = pmul(pfma(pneg(ch), abl, padd(pfma(pneg(ch), abh, sbh), sbl)), rabh);
-          P2 th, tl;
-          ptwo_sum(gh, ch, th, tl);
-          const P2 Kh = pneg(th), Kl = pneg(padd(padd(tl, gl), cl));
-          const P2 xr = newton_ff2(abh, abl, bh, bl, sbh, sbl, pneg(gh), pneg(gl), ch, cl, Kh, Kl,
-                                   make_float2(root[0], root[1]));
-          root[0] = xr.x;
-          root[1] = xr.y;
-        } else {
-          const F2 abf = two_sum(L.a1, -L.a2);
-          const float rabh = rcp32(abf.h);
-          const F2 fb1 = two_prod(L.b1, L.b1), fb2 = two_prod(L.b2, L.b2);
-          const F2 fg0 = two_sum(L.g, -L.a1), fg1 = two_sum(L.a2, -L.g);
-          // c = b2 / abar and K = -(g + c) as unnormalised pairs.
-          auto div_pair = [rabh, abf](const F2 num) {
-            const float q = num.h * rabh;
-            return F2{q, ((fmaf(-q, abf.h, num.h) + num.l) - q * abf.l) * rabh};
-          };
-          auto neg_sum_pair = [](const F2 a, const F2 b) {
-            const F2 t = two_sum(a.h, b.h);
-            return F2{-t.h, -((t.l + a.l) + b.l)};
-          };
-          const F2 fc0 = div_pair(fb2), fc1 = div_pair(fb1);
-          const F2 fK0 = neg_sum_pair(fg0, fc0), fK1 = neg_sum_pair(fg1, fc1);
-          root[0] = newton_ff(abf, fb1, fb2, fg0, fc0, fK0, root[0]);
-          root[1] = newton_ff(abf, fb2, fb1, fg1, fc1, fK1, root[1]);
-        }
-      }
-    }
+    // The warp's lanes that form eigenpairs (taken where all 32 are together),
+    // which rejoin after the class-specific part of the solve.
+    const unsigned fin_mask = __ballot_sync(0xffffffffu, L.cls != kIdle && L.cls != kNonFin);
+    float root[2];
+    const bool capped = roots_of<kComp>(L, root);
 
     bool flagged = false, nonfinite = false;
     int rk[3] = {0, 1, 2};  // rank of each eigenpair (ascending); identity for the other paths
@@ -730,10 +742,10 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
 #pragma unroll
         for (int k = 0; k < 9; ++k) U[k] = qnan;
       } else if (!kVectors) {
-        finish32_values<kMode == kPlain>(L, root[0], root[1], l, fin_mask);
+        finish32_values(L, root[0], root[1], l, fin_mask);
         unscale3(l, L.e);
       } else {
-        finish32<kMode != kInline>(L, root[0], root[1], l, U, rk, fin_mask);
+        finish32(L, root[0], root[1], l, U, rk, fin_mask);
         if (kComp && L.cls != kDiag) {
           // the eigenvalues' gaps in ascending order (min, median, max)
           const float lo = fminf(fminf(l[0], l[1]), l[2]), hi = fmaxf(fmaxf(l[0], l[1]), l[2]);
@@ -754,100 +766,26 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
       }
     }
 
-    if (kDefer) {
-      // Append the flagged lanes to the global list (one atomic per warp and
-      // class): reduced arrows from the front (count [0]), the other classes
-      // from the back (count [1]), so that k_refine_f32 runs each class in
-      // whole warps; it refines them and overwrites their outputs.
-      const bool fr = flagged && L.cls == kRed;
-      const unsigned mr = __ballot_sync(0xffffffffu, fr);
-      const unsigned mo = __ballot_sync(0xffffffffu, flagged && !fr);
-      unsigned long long br = 0, bo = 0;
-      if (lane_id == 0) {
-        if (mr) br = atomicAdd(&flag_count[0], (unsigned long long)__popc(mr));
-        if (mo) bo = atomicAdd(&flag_count[1], (unsigned long long)__popc(mo));
-      }
-      br = __shfl_sync(0xffffffffu, br, 0);
-      bo = __shfl_sync(0xffffffffu, bo, 0);
-      if (flagged) {
-        FlagRec r;
-        r.v[0] = L.a1; r.v[1] = L.a2; r.v[2] = L.b1; r.v[3] = L.b2; r.v[4] = L.g; r.v[5] = L.c; r.v[6] = L.s;
-        r.v[7] = root[0]; r.v[8] = root[1];
-        r.code = (L.e << 2) | L.cls;
-        r.gidx = base + tid;
-        const int64_t at = fr ? (int64_t)(br + __popc(mr & lt_mask)) : n - 1 - (int64_t)(bo + __popc(mo & lt_mask));
-        flag_list[at] = r;
-      }
-    } else if (kComp) {
-      // Compact the flagged lanes after the carried ones and refine a whole
-      // number of warps' worth of them in FP64, with every lane of the CTA
-      // available; the rest (fewer than 32) are carried to the next tile, so
-      // no warp runs the FP64 code with idle lanes.  A lane of this tile
-      // gets its refined result in the staging area, a carried one straight
-      // in memory (over the FP32 result written with its own tile).  The
-      // CTA refines its last carried lanes after its final tile.
+    if constexpr (kComp) {
       const unsigned m = __ballot_sync(0xffffffffu, flagged);
-      int wbase = 0;
-      if (lane_id == 0 && m) wbase = atomicAdd(&s_nflag, __popc(m));
-      wbase = __shfl_sync(0xffffffffu, wbase, 0);
-      if (flagged) {
-        const int slot = nfc + wbase + __popc(m & lt_mask);
-        float* f = &s_fa[slot * kFA];
-        f[0] = L.a1; f[1] = L.a2; f[2] = L.b1; f[3] = L.b2; f[4] = L.g; f[5] = L.c; f[6] = L.s;
-        f[7] = root[0]; f[8] = root[1];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) f[9 + k] = a_in[k];
-        s_fc[slot] = (L.e << 2) | L.cls;
-        if constexpr (kServe) {
-          const TileRef<float> r = s_ref[buf];
-          s_fg[slot] = (int64_t)reinterpret_cast<uintptr_t>(r.lam + tid * 3);
-          s_fU[slot] = r.U ? r.U + tid * 9 : nullptr;
-        } else {
-          s_fg[slot] = base + tid;
+      const int before = __popc(m & ((1u << lane_id) - 1u));
+      if constexpr (kList) {
+        int at = 0;
+        if (lane_id == 0 && m) at = atomicAdd(&s_nflag, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + before;
+        if (flagged) {
+          if constexpr (kServe)
+            s_list.at[at] =
+                TileRef<float>{s_ref[buf].src + tid * 6, lam_tile + tid * 3, want_U ? U_tile + tid * 9 : nullptr, 1};
+          else
+            s_list.seq[at] = seq;
         }
+      } else {
+        unsigned long long at = 0;
+        if (lane_id == 0 && m) at = atomicAdd(flag_count, (unsigned long long)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (flagged) flag_list[at + before] = base + tid;
       }
-      __syncthreads();
-      const int n_avail = nfc + s_nflag;
-      const int P = n_avail & ~31;
-      for (int i = tid; i < P; i += kTPB) {
-        double lam[3], U[9];
-        // The residual check (counter [3]) only when counters are asked for.
-        const bool bad = refine_one(&s_fa[i * kFA], s_fc[i], counters != nullptr ? &s_fa[i * kFA + 9] : nullptr,
-                                    lam, U);
-        if (bad) atomicAdd(&counters[3], 1ull);
-        const int64_t gi = s_fg[i];
-        int64_t row;
-        float *dl_far, *dU_far;  // where a lane of an earlier tile writes
-        if constexpr (kServe) {
-          const int64_t d = (int64_t)(uintptr_t)gi - (int64_t)reinterpret_cast<uintptr_t>(s_ref[buf].lam);
-          row = (d >= 0 && d < (int64_t)cnt * 12) ? d / 12 : -1;
-          dl_far = reinterpret_cast<float*>((uintptr_t)gi);
-          dU_far = s_fU[i];
-        } else {
-          row = gi - base;
-          dl_far = lam_out + gi * 3;
-          dU_far = want_U ? U_out + gi * 9 : nullptr;
-        }
-        const bool here = row >= 0 && row < cnt;
-        float* dl = here ? &s_lam[row * 3] : dl_far;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) dl[k] = (float)lam[k];
-        if (here || dU_far != nullptr) {
-          float* dU = here ? &s_U[row * 9] : dU_far;
-#pragma unroll
-          for (int k = 0; k < 9; ++k) dU[k] = (float)U[k];
-        }
-      }
-      __syncthreads();
-      const int nc_next = n_avail - P;
-      if (P > 0 && tid < nc_next) {  // [P, n_avail) -> [0, nc_next): no overlap, P >= 32 > nc_next
-#pragma unroll
-        for (int k = 0; k < kFA; ++k) s_fa[tid * kFA + k] = s_fa[(P + tid) * kFA + k];
-        s_fc[tid] = s_fc[P + tid];
-        s_fg[tid] = s_fg[P + tid];
-        if constexpr (kServe) s_fU[tid] = s_fU[P + tid];
-      }
-      nfc = nc_next;
     }
     if (counters != nullptr) {
       const unsigned cm = __ballot_sync(0xffffffffu, capped);
@@ -859,51 +797,57 @@ __global__ void __launch_bounds__(kTPB) k_syev3_f32(const float* __restrict__ A,
         if (fl) atomicAdd(&counters[2], (unsigned long long)__popc(fl));
       }
     }
+    fence_async_shared();
     __syncthreads();
-    if (tid == 0) s_nflag = 0;
 
-    {
-      float* dst = kServe ? s_ref[buf].lam : lam_out + base * 3;
-      const int m = cnt * 3;
-      if (vec_lam) {
-        float4* d4 = reinterpret_cast<float4*>(dst);
-        const float4* s4 = reinterpret_cast<const float4*>(s_lam);
-        for (int i = tid; i < m / 4; i += kTPB) d4[i] = s4[i];
-        for (int i = (m & ~3) + tid; i < m; i += kTPB) dst[i] = s_lam[i];
-      } else {
-        for (int i = tid; i < m; i += kTPB) dst[i] = s_lam[i];
+    // A full, aligned tile's rows leave by bulk copy; the staging area is
+    // written again only after thread 0 has seen it read (above, before the
+    // next tile's barrier).
+    if (cnt == kTPB && vec_lam && (!want_U || vec_U)) {
+      if (tid == 0) {
+        bulk_s2g(lam_tile, s_lam, kTPB * 12);
+        if (kVectors && want_U) bulk_s2g(U_tile, s_U, kTPB * 36);
       }
+    } else {
+      auto store = [&](float* dst, const float* src, const int m, const bool vec) {
+        const int m4 = vec ? m / 4 : 0;
+        for (int i = tid; i < m4; i += kTPB)
+          reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
+        for (int i = 4 * m4 + tid; i < m; i += kTPB) dst[i] = src[i];
+      };
+      store(lam_tile, s_lam, cnt * 3, vec_lam);
+      if (kVectors && want_U) store(U_tile, s_U, cnt * 9, vec_U);
     }
-    if (want_U) {
-      float* dst = kServe ? s_ref[buf].U : U_out + base * 9;
-      const int m = cnt * 9;
-      if (vec_U) {
-        float4* d4 = reinterpret_cast<float4*>(dst);
-        const float4* s4 = reinterpret_cast<const float4*>(s_U);
-        for (int i = tid; i < m / 4; i += kTPB) d4[i] = s4[i];
-        for (int i = (m & ~3) + tid; i < m; i += kTPB) dst[i] = s_U[i];
-      } else {
-        for (int i = tid; i < m; i += kTPB) dst[i] = s_U[i];
-      }
+    if constexpr (kList) {
+      if (s_nflag > kCap - kTPB) refine();  // (s_nflag is stable between the tiles' barriers)
     }
-    __syncthreads();
   }
-  if (kInl) {
-    // The flagged lanes still carried after the CTA's final tile (nfc is
-    // CTA-uniform; the list was completed before the loop's last barrier).
-    for (int i = tid; i < nfc; i += kTPB) {
-      double lam[3], U[9];
-      const bool bad = refine_one(&s_fa[i * kFA], s_fc[i], counters != nullptr ? &s_fa[i * kFA + 9] : nullptr,
-                                  lam, U);
-      if (bad) atomicAdd(&counters[3], 1ull);
-      const int64_t gi = s_fg[i];
-      float* dl = kServe ? reinterpret_cast<float*>((uintptr_t)gi) : lam_out + gi * 3;
-      float* dU = kServe ? s_fU[kServe ? i : 0] : (want_U ? U_out + gi * 9 : nullptr);
+  if constexpr (kList) refine();
+  if (tid == 0) bulk_read_wait();
+}
+
+// The refinement of the deferred form: the listed matrices, in whole warps.
+__global__ void __launch_bounds__(kTPB, 5) k_refine_list(const int64_t* __restrict__ rows,
+                                                         const unsigned long long* __restrict__ count,
+                                                         const float* __restrict__ A, float* __restrict__ lam_out,
+                                                         float* __restrict__ U_out,
+                                                         unsigned long long* __restrict__ counters) {
+  const int64_t m = (int64_t)*count;
+  const int lane_id = threadIdx.x & 31;
+  for (int64_t i0 = (int64_t)blockIdx.x * kTPB + (threadIdx.x & ~31u); i0 < m; i0 += (int64_t)gridDim.x * kTPB) {
+    const bool active = i0 + lane_id < m;
+    const int64_t row = rows[active ? i0 + lane_id : m - 1];
+    float rec[6], out[12];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) dl[k] = (float)lam[k];
-      if (dU != nullptr) {
+    for (int k = 0; k < 6; ++k) rec[k] = A[row * 6 + k];
+    const bool bad = refine_record(rec, active, counters != nullptr, out);
+    if (bad) atomicAdd(&counters[3], 1ull);
+    if (active) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dU[k] = (float)U[k];
+      for (int k = 0; k < 3; ++k) lam_out[row * 3 + k] = out[k];
+      if (U_out != nullptr) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) U_out[row * 9 + k] = out[3 + k];
       }
     }
   }
@@ -921,19 +865,13 @@ int blocks_per_sm_f32() {
   return cached;
 }
 
-// per_sm_cap > 0: at most that many CTAs per SM (room left for a kernel
-// that runs beside this one).
 template <bool kBulkIn, int kMode, bool kVectors = true>
-cudaError_t launch(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters,
-                   FlagRec* flag_list, unsigned long long* flag_count, cudaStream_t stream, int sms,
-                   int per_sm_cap = 0) {
+cudaError_t launch(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters, cudaStream_t stream,
+                   int sms, int64_t* flag_list = nullptr, unsigned long long* flag_count = nullptr) {
   const int64_t n_tiles = (n + kTPB - 1) / kTPB;
-  int per_sm = blocks_per_sm_f32<kBulkIn, kMode, kVectors>();
-  if (per_sm_cap > 0 && per_sm > per_sm_cap) per_sm = per_sm_cap;
-  const int64_t resident = (int64_t)sms * per_sm;
+  const int64_t resident = (int64_t)sms * blocks_per_sm_f32<kBulkIn, kMode, kVectors>();
   const int grid = (int)(n_tiles < resident ? n_tiles : resident);
-  k_syev3_f32<kBulkIn, kMode, kVectors>
-      <<<grid, kTPB, 0, stream>>>(A, n, lam, U, counters, flag_list, flag_count, nullptr);
+  k_syev3_f32<kBulkIn, kMode, kVectors><<<grid, kTPB, 0, stream>>>(A, n, lam, U, counters, flag_list, flag_count, nullptr);
   return cudaGetLastError();
 }
 
@@ -942,46 +880,8 @@ cudaError_t launch_serve(const ServeList* list, unsigned long long* counters, cu
   // The list's length is known only on the device: a resident grid; CTAs
   // without a tile exit at once.
   const int grid = sms * blocks_per_sm_f32<true, kMode, true, true>();
-  k_syev3_f32<true, kMode, true, true>
-      <<<grid, kTPB, 0, stream>>>(nullptr, 0, nullptr, nullptr, counters, nullptr, nullptr, list);
+  k_syev3_f32<true, kMode, true, true><<<grid, kTPB, 0, stream>>>(nullptr, 0, nullptr, nullptr, counters, nullptr, nullptr, list);
   return cudaGetLastError();
-}
-
-// The refinement of the deferred compensated form: one flagged lane per
-// thread, grid-stride over the list (its lengths are read on the device):
-// first the reduced arrows (list front), then the other classes (list back,
-// n records from the front), so each warp but one runs a single class.
-constexpr int kRefineTPB = 128;
-
-__global__ void __launch_bounds__(kRefineTPB) k_refine_f32(const FlagRec* __restrict__ list,
-                                                           const unsigned long long* __restrict__ count,
-                                                           int64_t n, const float* __restrict__ A,
-                                                           float* __restrict__ lam_out, float* __restrict__ U_out,
-                                                           unsigned long long* __restrict__ counters) {
-  const unsigned long long m_red = count[0], m = m_red + count[1];
-  for (unsigned long long i = (unsigned long long)blockIdx.x * kRefineTPB + threadIdx.x; i < m;
-       i += (unsigned long long)gridDim.x * kRefineTPB) {
-    const FlagRec r = list[i < m_red ? (int64_t)i : n - 1 - (int64_t)(i - m_red)];
-    double lam[3], U[9];
-    const bool bad = refine_one(r.v, r.code, counters != nullptr ? A + r.gidx * 6 : nullptr, lam, U);
-    if (bad) atomicAdd(&counters[3], 1ull);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) lam_out[r.gidx * 3 + k] = (float)lam[k];
-    if (U_out != nullptr) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) U_out[r.gidx * 9 + k] = (float)U[k];
-    }
-  }
-}
-
-int refine_blocks_per_sm() {
-  static int cached = -1;
-  if (cached < 0) {
-    int v = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_refine_f32, kRefineTPB, 0);
-    cached = (e == cudaSuccess && v > 0) ? v : 1;
-  }
-  return cached;
 }
 
 }  // namespace
@@ -995,13 +895,41 @@ cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool com
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const bool bulk = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-  if (bulk && !compensated && U == nullptr)
-    return launch<true, kPlain, false>(A, n, lam, U, counters, nullptr, nullptr, stream, sms);
-  if (bulk)
-    return compensated ? launch<true, kInline>(A, n, lam, U, counters, nullptr, nullptr, stream, sms)
-                       : launch<true, kPlain>(A, n, lam, U, counters, nullptr, nullptr, stream, sms);
-  return compensated ? launch<false, kInline>(A, n, lam, U, counters, nullptr, nullptr, stream, sms)
-                     : launch<false, kPlain>(A, n, lam, U, counters, nullptr, nullptr, stream, sms);
+  if (compensated)
+    return bulk ? launch<true, kComp32>(A, n, lam, U, counters, stream, sms)
+                : launch<false, kComp32>(A, n, lam, U, counters, stream, sms);
+  if (bulk && U == nullptr) return launch<true, kPlain, false>(A, n, lam, U, counters, stream, sms);
+  return bulk ? launch<true, kPlain>(A, n, lam, U, counters, stream, sms)
+              : launch<false, kPlain>(A, n, lam, U, counters, stream, sms);
+}
+
+// From this size on the workspace form lists its flagged matrices there and
+// refines them with a second kernel: the solve then needs 64 registers instead
+// of 80 (8 CTAs per SM instead of 6), which pays for the second launch and the
+// list.  Measured, us, this form against the single kernel: 2^23 matrices with
+// 4 % flagged 363 / 412, none flagged 258 / 277; 2^21: 97 / 114, 76 / 72; 2^20:
+// 58 / 68, 45 / 42.  (The earlier form, the refinement by FP64 code on a second
+// stream beside the solve: 414 at 2^23.)
+constexpr int64_t kDeferMin = (int64_t)1 << 21;
+
+cudaError_t launch_f32c_ws(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters, void* work,
+                           cudaStream_t stream) {
+  if (n < kDeferMin) return launch_f32(A, n, lam, U, true, counters, stream);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  auto* count = static_cast<unsigned long long*>(work);
+  auto* rows = reinterpret_cast<int64_t*>(static_cast<char*>(work) + kFlagListOffset);
+  e = cudaMemsetAsync(count, 0, sizeof(*count), stream);
+  if (e != cudaSuccess) return e;
+  e = (reinterpret_cast<uintptr_t>(A) & 15) == 0
+          ? launch<true, kDeferred>(A, n, lam, U, counters, stream, sms, rows, count)
+          : launch<false, kDeferred>(A, n, lam, U, counters, stream, sms, rows, count);
+  if (e != cudaSuccess) return e;
+  k_refine_list<<<sms * 5, kTPB, 0, stream>>>(rows, count, A, lam, U, counters);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_f32_serve(const ServeList* list, bool compensated, unsigned long long* counters,
@@ -1011,117 +939,8 @@ cudaError_t launch_f32_serve(const ServeList* list, bool compensated, unsigned l
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  return compensated ? launch_serve<kInline>(list, counters, stream, sms)
+  return compensated ? launch_serve<kComp32>(list, counters, stream, sms)
                      : launch_serve<kPlain>(list, counters, stream, sms);
-}
-
-size_t f32c_workspace_bytes(int64_t n) { return kFlagListOffset + (size_t)n * sizeof(FlagRec); }
-
-namespace {
-
-// Pipelined deferred path: a batch of at least kPipeMin matrices is cut into
-// kPipeChunks runs of whole tiles; the FP32 kernel solves the runs one after
-// the other on the caller's stream, and the refinement of run c starts on a
-// side stream (after an event recorded behind run c's FP32 kernel) while the
-// FP32 kernel works on run c + 1.  The FP32 grid leaves room for
-// kPipeRefinePerSM refinement CTAs on every SM, so the refinement -- bound by
-// the FP64 pipe -- runs beside the FP32 solve, which is bound by instruction
-// issue.  The caller's stream waits for the side stream at the end.  The
-// side stream and the events are created once per device, and one call's
-// records and waits are enqueued under a lock so that calls from several
-// host threads do not interleave them.
-constexpr int64_t kPipeMin = (int64_t)1 << 21;
-constexpr int kPipeChunks = 8;        // counters: 2 per run, 16 B x 8 <= kFlagListOffset
-// Refinement CTAs per SM beside the FP32 kernel (measured on the 2^24 mixed
-// batch: 1, 2, 3, 4, 5, 6 gave 1.39, 1.33, 1.59, 1.53, 1.54, 1.48e10
-// eigensolves/s; 16 runs instead of 8 were slower, 4 the same; without the
-// pipeline 1.37e10).  With 3, the register file holds 9 FP32 CTAs and 2
-// refinement CTAs per SM.
-constexpr int kPipeRefinePerSM = 3;
-static_assert(2 * sizeof(unsigned long long) * kPipeChunks <= kFlagListOffset, "run counters fit");
-constexpr int kPipeMaxDevices = 64;
-
-struct Pipe {
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev[kPipeChunks + 1] = {};
-};
-std::mutex g_pipe_mu;
-Pipe g_pipe[kPipeMaxDevices];
-
-cudaError_t pipe_for(int dev, Pipe** out) {
-  Pipe& P = g_pipe[dev];
-  if (P.side == nullptr) {
-    cudaStream_t s = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    for (int i = 0; i <= kPipeChunks; ++i) {
-      e = cudaEventCreateWithFlags(&P.ev[i], cudaEventDisableTiming);
-      if (e != cudaSuccess) {
-        for (int j = 0; j < i; ++j) cudaEventDestroy(P.ev[j]);
-        cudaStreamDestroy(s);
-        return e;
-      }
-    }
-    P.side = s;
-  }
-  *out = &P;
-  return cudaSuccess;
-}
-
-}  // namespace
-
-cudaError_t launch_f32c_deferred(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters,
-                                 void* work, cudaStream_t stream) {
-  if (n <= 0) return cudaSuccess;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  auto* count = static_cast<unsigned long long*>(work);
-  auto* list = reinterpret_cast<FlagRec*>(static_cast<char*>(work) + kFlagListOffset);
-  const bool bulk = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-  if (n < kPipeMin || dev < 0 || dev >= kPipeMaxDevices) {
-    e = cudaMemsetAsync(count, 0, 2 * sizeof(unsigned long long), stream);
-    if (e != cudaSuccess) return e;
-    e = bulk ? launch<true, kDeferred>(A, n, lam, U, counters, list, count, stream, sms)
-             : launch<false, kDeferred>(A, n, lam, U, counters, list, count, stream, sms);
-    if (e != cudaSuccess) return e;
-    k_refine_f32<<<sms * refine_blocks_per_sm(), kRefineTPB, 0, stream>>>(list, count, n, A, lam, U, counters);
-    return cudaGetLastError();
-  }
-  std::lock_guard<std::mutex> hold(g_pipe_mu);
-  Pipe* P = nullptr;
-  e = pipe_for(dev, &P);
-  if (e != cudaSuccess) return e;
-  // Runs of whole tiles (128 matrices: every run starts 16-byte aligned in
-  // all three arrays when the batch does); run c uses counters [2c, 2c+1]
-  // and the list records [start, start + len) of its own matrices.
-  const int64_t len = ((n + kPipeChunks - 1) / kPipeChunks + kTPB - 1) / kTPB * kTPB;
-  e = cudaMemsetAsync(count, 0, 2 * sizeof(unsigned long long) * kPipeChunks, stream);
-  if (e != cudaSuccess) return e;
-  const int cap = blocks_per_sm_f32<true, kDeferred, true>() - kPipeRefinePerSM;
-  for (int c = 0; c < kPipeChunks; ++c) {
-    const int64_t start = c * len;
-    if (start >= n) break;
-    const int64_t m = (n - start) < len ? (n - start) : len;
-    const float* Ac = A + start * 6;
-    float* lc = lam + start * 3;
-    float* Uc = U ? U + start * 9 : nullptr;
-    unsigned long long* cc = count + 2 * c;
-    e = bulk ? launch<true, kDeferred>(Ac, m, lc, Uc, counters, list + start, cc, stream, sms, cap > 0 ? cap : 1)
-             : launch<false, kDeferred>(Ac, m, lc, Uc, counters, list + start, cc, stream, sms, cap > 0 ? cap : 1);
-    if (e != cudaSuccess) return e;
-    e = cudaEventRecord(P->ev[c], stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(P->side, P->ev[c], 0);
-    if (e != cudaSuccess) return e;
-    k_refine_f32<<<sms * kPipeRefinePerSM, kRefineTPB, 0, P->side>>>(list + start, cc, m, Ac, lc, Uc, counters);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  e = cudaEventRecord(P->ev[kPipeChunks], P->side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, P->ev[kPipeChunks], 0);
-  return e;
 }
 
 cudaError_t take_flags_f32(unsigned* flags) {

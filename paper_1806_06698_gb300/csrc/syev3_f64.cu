@@ -68,17 +68,6 @@ __device__ __forceinline__ void diagonal(const double a[6], double l[3], double 
   rk[2] = (int)(k0 <= k2) + (int)(k1 <= k2);
 }
 
-// Sign rule of column k of U: its largest-magnitude component, the first of
-// equals, becomes positive (magnitudes compared as integers, sign bits
-// flipped).
-__device__ __forceinline__ void sign_rule(double U[9], const int k) {
-  const uint64_t m0 = mag_bits(U[k]), m1 = mag_bits(U[3 + k]), m2 = mag_bits(U[6 + k]);
-  const double big = (m2 > m0 && m2 > m1) ? U[6 + k] : ((m1 > m0) ? U[3 + k] : U[k]);
-  const int flip = __double2hiint(big) & (int)0x80000000;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) U[i * 3 + k] = flip_sign(U[i * 3 + k], flip);
-}
-
 // kVectors = false: eigenvalues only (U_out is NULL).
 // kServe: the serving build.  The tiles are those of the device-resident
 // work list `list` (A, n, lam_out and U_out are unused): runs of matrices of
@@ -232,7 +221,7 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
         } else if (F.similar && fx::solve<kVectors>(F, l, U, rk)) {
           if (kVectors) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) sign_rule(U, k);
+            for (int k = 0; k < 3; ++k) fx::sign_rule(U, k);
           }
         } else {
           left = true;

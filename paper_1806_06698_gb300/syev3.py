@@ -123,7 +123,7 @@ def syev3_batched(A6: torch.Tensor, *, vectors: bool = True, compensated: bool =
     optional uint64-sized (int64) device tensor of 4 entries the kernels add
     to (see include/syev3.h).  ``workspace`` (a device tensor of at least
     workspace_bytes(...) bytes) selects syev3_batched_ws: for the compensated
-    form, the FP64 refinement as a second kernel."""
+    form and large batches, the refinement as a second kernel."""
     if not A6.is_cuda:
         raise ValueError("A6 must be a CUDA tensor (no CPU fallback)")
     if A6.dim() != 2 or A6.shape[1] != 6 or not A6.is_contiguous():
@@ -175,16 +175,15 @@ def syev3_batched_method(A6: torch.Tensor, *, zero_finder: int = ZF_PRODUCTION,
     return lam, U
 
 
-# Largest batch of syev3_batched_static_ws (its scratch is a static array).
+# Largest batch of syev3_batched_static_ws (include/syev3.h).
 STATIC_MAX_N = 262144
 
 
 def syev3_batched_static_ws(A6: torch.Tensor, *, vectors: bool = True,
                             out: tuple[torch.Tensor, torch.Tensor | None] | None = None,
                             counters: torch.Tensor | None = None, stream=None):
-    """The compensated FP32 solve with its refinement list in the library's
-    static device memory (no workspace, no allocation); n <= STATIC_MAX_N.
-    Calls on one device must not overlap in time."""
+    """The compensated FP32 solve without a workspace or an allocation of the
+    library's own; n <= STATIC_MAX_N."""
     if not A6.is_cuda or A6.dtype != torch.float32:
         raise ValueError("A6 must be a float32 CUDA tensor (no CPU fallback)")
     if A6.dim() != 2 or A6.shape[1] != 6 or not A6.is_contiguous():
