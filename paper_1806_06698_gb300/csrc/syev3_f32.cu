@@ -570,7 +570,7 @@ struct FlagList<true> {
 // its start is not 16-byte aligned.  The production builds (kServe = false)
 // compile this out.
 template <bool kBulkIn, int kMode, bool kVectors = true, bool kServe = false>
-__global__ void __launch_bounds__(kTPB, kMode == kComp32 ? 6 : 1)
+__global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32 ? 6 : 8))
     k_syev3_f32(const float* __restrict__ A, int64_t n, float* __restrict__ lam_out, float* __restrict__ U_out,
                 unsigned long long* __restrict__ counters, int64_t* __restrict__ flag_list,
                 unsigned long long* __restrict__ flag_count, const ServeList* __restrict__ list) {
