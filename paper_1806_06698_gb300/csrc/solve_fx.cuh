@@ -130,28 +130,47 @@ __device__ __forceinline__ void rotation(const Quat q, int64_t R[9], int64_t& no
   R[7] = madw(w2, q.x, 2 * yz);
 }
 
-// R^T (A/2) R x 2^61 (upper triangle 00 01 11 02 12 22); a holds the limbs of
-// the packed A/2 (11, 22, 33, 12, 13, 23) x 2^62.
-__device__ __forceinline__ void rotated(const Split a[6], const Split r[9], int64_t B[6]) {
+// (A/2) b for a column b of R, x 2^61.
+__device__ __forceinline__ void times_column(const Split a[6], const Split b0, const Split b1, const Split b2,
+                                             Split t[3]) {
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    Split t[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const Split a0 = i == 0 ? a[0] : (i == 1 ? a[3] : a[4]);
-      const Split a1 = i == 0 ? a[3] : (i == 1 ? a[1] : a[5]);
-      const Split a2 = i == 0 ? a[4] : (i == 1 ? a[5] : a[2]);
-      int64_t hh, cross = 1ll << 29;  // half a unit (the l l terms' signs are those of a)
-      dot3(a0, a1, a2, r[j], r[3 + j], r[6 + j], hh, cross);
-      t[i] = split31((hh << 1) + (cross >> 30));
-    }
-#pragma unroll
-    for (int i = 0; i <= j; ++i) {
-      int64_t hh, cross = 0x70000000ll;  // mean of the l l terms (3 x 2^29) and half a unit
-      dot3(t[0], t[1], t[2], r[i], r[3 + i], r[6 + i], hh, cross);
-      B[j * (j + 1) / 2 + i] = (hh << 2) + (cross >> 29);
-    }
+  for (int i = 0; i < 3; ++i) {
+    const Split a0 = i == 0 ? a[0] : (i == 1 ? a[3] : a[4]);
+    const Split a1 = i == 0 ? a[3] : (i == 1 ? a[1] : a[5]);
+    const Split a2 = i == 0 ? a[4] : (i == 1 ? a[5] : a[2]);
+    int64_t hh, cross = 1ll << 29;  // half a unit (the l l terms' signs are those of a)
+    dot3(a0, a1, a2, b0, b1, b2, hh, cross);
+    t[i] = split31((hh << 1) + (cross >> 30));
   }
+}
+
+__device__ __forceinline__ int64_t dot_column(const Split r0, const Split r1, const Split r2, const Split t[3]) {
+  int64_t hh, cross = 0x70000000ll;  // mean of the l l terms (3 x 2^29) and half a unit
+  dot3(t[0], t[1], t[2], r0, r1, r2, hh, cross);
+  return (hh << 2) + (cross >> 29);
+}
+
+// R^T (A/2) R x 2^61 (upper triangle 00 01 11 02 12 22); a holds the limbs of
+// the packed A/2 (11, 22, 33, 12, 13, 23) x 2^62, r those of R, 1 + eta times a
+// rotation (norm = 2^60 (1 + eta)); trace: that of A/2 x 2^61.  The third diagonal entry is the trace's remainder -- R^T A R has the
+// trace (1 + eta)^2 tr A -- so that only two of A R's columns are formed: 11
+// products of three terms instead of 15.
+__device__ __forceinline__ void rotated(const Split a[6], const Split r[9], const int64_t trace, const int64_t norm,
+                                        int64_t B[6]) {
+  Split t[3];
+  times_column(a, r[0], r[3], r[6], t);
+  B[0] = dot_column(r[0], r[3], r[6], t);
+  B[3] = dot_column(r[2], r[5], r[8], t);
+  times_column(a, r[1], r[4], r[7], t);
+  B[1] = dot_column(r[0], r[3], r[6], t);
+  B[2] = dot_column(r[1], r[4], r[7], t);
+  B[4] = dot_column(r[2], r[5], r[8], t);
+  const int64_t eta = norm - (1ll << 60);  // below 2^40
+  const float etaf = to_float(eta);
+  const int64_t both = 2 * eta + (int64_t)__float2int_rn(etaf * etaf * 0x1p-60f);  // (1 + eta)^2 - 1, x 2^60
+  const Split T = split31(trace), E = split31(both);
+  const int64_t grow = ((int64_t)T.h * E.h << 2) + (madw(T.h, E.l, (int64_t)T.l * E.h) >> 29);
+  B[5] = trace + grow - B[0] - B[2];
 }
 
 // The eigenvector frame of a (|a| < 1) by the FP32 method: outer
@@ -364,21 +383,19 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   Quat q = {__float2int_rn(f.w * sc), __float2int_rn(f.x * sc), __float2int_rn(f.y * sc), __float2int_rn(f.z * sc)};
   int64_t R[9], N, B[6];
   Split Rs[9];
+  // trace of A/2 x 2^61
+  const int64_t trace = (((int64_t)As[0].h + As[1].h + As[2].h) << 30) + (((int64_t)As[0].l + As[1].l + As[2].l) >> 1);
   rotation(q, R, N);
 #pragma unroll
   for (int i = 0; i < 9; ++i) Rs[i] = split31(R[i]);
-  rotated(As, Rs, B);
+  rotated(As, Rs, trace, N, B);
   int p[3];
   small_rotation(B, p);
   q = normalised(times(q, p));
   rotation(q, R, N);
-  const int eta = (int)((N - (1ll << 60)) >> 2);  // eta x 2^58
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    R[i] -= ((int64_t)(int)(R[i] >> 31) * eta) >> 27;
-    Rs[i] = split31(R[i]);
-  }
-  rotated(As, Rs, B);
+  for (int i = 0; i < 9; ++i) Rs[i] = split31(R[i]);
+  rotated(As, Rs, trace, N, B);
   float e01 = to_float(B[1]), e02 = to_float(B[3]), e12 = to_float(B[4]);
   const float off = fmaxf(fabsf(e01), fmaxf(fabsf(e02), fabsf(e12)));
   float w01 = quotient(e01, to_float(B[2] - B[0])), w02 = quotient(e02, to_float(B[5] - B[0])),
@@ -394,28 +411,42 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   rk[0] = (int)(B[2] < B[0]) + (int)(B[5] < B[0]);
   rk[1] = (int)(B[0] <= B[2]) + (int)(B[5] < B[2]);
   rk[2] = (int)(B[0] <= B[5]) + (int)(B[2] <= B[5]);
-  l[0] = to_double_int<60>(B[0], F.e);
-  l[1] = to_double_int<60>(B[2], F.e);
-  l[2] = to_double_int<60>(B[5], F.e);
+  // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
+  // and, with the perturbation below, R by 1 + eta.
+  const int eta = (int)((N - (1ll << 60)) >> 3);                    // x 2^57
+  const int shrink = eta - 3 * (int)(((int64_t)eta * eta) >> 58);  // eta - 3/2 eta^2
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int64_t b = k == 0 ? B[0] : (k == 1 ? B[2] : B[5]);
+    l[k] = to_double_int<60>(b - (((int64_t)(int)(b >> 31) * shrink) >> 25), F.e);
+  }
   if (kVectors) {
-    // R (I + W + W^2/2), W antisymmetric: orthogonal to third order.
-    const int x01 = __float2int_rn(w01 * 0x1p53f), x02 = __float2int_rn(w02 * 0x1p53f),
-              x12 = __float2int_rn(w12 * 0x1p53f);
+    // R (I + W + W^2/2 - eta), W antisymmetric: orthogonal to third order.  The
+    // factors are held x 2^57 when W is small enough, as it is but for close
+    // pairs, else x 2^53.
+    const bool fine = big <= 0x1p-27f;
+    const float c = fine ? 0x1p57f : 0x1p53f, hc = 0.5f * c;
+    const int x01 = __float2int_rn(w01 * c), x02 = __float2int_rn(w02 * c), x12 = __float2int_rn(w12 * c);
+    const int scale = fine ? eta : (eta + 8) >> 4;
     const float s02 = w02 * w02, s12 = w12 * w12;
-    const int n0 = __float2int_rn(-0x1p52f * fmaf(w01, w01, s02)), n1 = __float2int_rn(-0x1p52f * fmaf(w01, w01, s12)),
-              n2 = __float2int_rn(-0x1p52f * fmaf(w02, w02, s12));
-    const int y01 = __float2int_rn(-0x1p52f * w02 * w12), y02 = __float2int_rn(0x1p52f * w01 * w12),
-              y12 = __float2int_rn(-0x1p52f * w01 * w02);
+    const int n0 = __float2int_rn(-hc * fmaf(w01, w01, s02)) - scale,
+              n1 = __float2int_rn(-hc * fmaf(w01, w01, s12)) - scale,
+              n2 = __float2int_rn(-hc * fmaf(w02, w02, s12)) - scale;
+    const int y01 = __float2int_rn(-hc * w02 * w12), y02 = __float2int_rn(hc * w01 * w12),
+              y12 = __float2int_rn(-hc * w01 * w02);
+    const int shift = fine ? 25 : 21;
+    const int64_t half = 1ll << (shift - 1);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const int r0 = Rs[3 * i].h, r1 = Rs[3 * i + 1].h, r2 = Rs[3 * i + 2].h;  // x 2^29
-      constexpr int64_t half = 1ll << 20;
-      const int64_t d0 = madw(r2, y02 - x02, madw(r1, y01 - x01, madw(r0, n0, half)));  // x 2^82
+      const int64_t d0 = madw(r2, y02 - x02, madw(r1, y01 - x01, madw(r0, n0, half)));
       const int64_t d1 = madw(r2, y12 - x12, madw(r1, n1, madw(r0, y01 + x01, half)));
       const int64_t d2 = madw(r2, n2, madw(r1, y12 + x12, madw(r0, y02 + x02, half)));
-      U[i * 3 + 0] = to_double_int<61>((R[3 * i] << 1) + (d0 >> 21));
-      U[i * 3 + 1] = to_double_int<61>((R[3 * i + 1] << 1) + (d1 >> 21));
-      U[i * 3 + 2] = to_double_int<61>((R[3 * i + 2] << 1) + (d2 >> 21));
+      U[i * 3 + 0] = to_double_int<61>((R[3 * i] << 1) + (d0 >> shift));
+      U[i * 3 + 1] = to_double_int<61>((R[3 * i + 1] << 1) + (d1 >> shift));
+      // a third of the conversions on the otherwise idle FP64 pipe (2^22 mixed
+      // matrices 522 us, none 530, two thirds 544)
+      U[i * 3 + 2] = to_double<61>((R[3 * i + 2] << 1) + (d2 >> shift));
     }
   }
   return true;
