@@ -13,18 +13,20 @@
 //  * matrices left to the FP64 path are gathered from tile to tile and solved
 //    kTPB at a time, so that each of the SM's FP64 units works on full warps
 //    while the SM's other CTA is in the integer part;
-//  * there, both shifted roots are located in FP32, moved right of the root
-//    by a bound on the FP32 error and finished by one FP64 Borges-Gragg step
-//    and the paper's stopping test; the roots that do not pass are compacted
-//    with warp ballots and finished by the full FP64 iteration.
+//  * there, a matrix whose couplings are far below every gap of its diagonal
+//    takes second-order perturbation (33 FP64 operations); for the others both
+//    shifted roots are located in FP32, moved right of the root by a bound on
+//    the FP32 error and finished by one FP64 Borges-Gragg step and the paper's
+//    stopping test; the roots that do not pass are compacted with warp ballots
+//    and finished by the full FP64 iteration.
 //
-// Measured (ncu, 2^22 well-separated matrices): 2650 thread instructions per
-// matrix, issue slots 52 % used, the integer and FMA pipes each about 50 %,
-// the FP64 pipe 6 %; no one unit is full, the dependent chains of 16 warps per
-// SM and instruction fetch (see kTile) are what is left.  2^24 mixed matrices
-// (11 % of them on the FP64 path): 2.59 ms, against 6.39 ms when every matrix
-// took the FP64 path (FP64 pipe 83 % busy); eigenvalues only, 10^6: 131 us
-// against 292.
+// Measured (ncu, 2^22 well-separated matrices): 2370 thread instructions per
+// matrix, issue slots 56 % used, the integer and FMA pipes each about 53 %,
+// the FP64 pipe idle; no one unit is full, more resident warps change nothing
+// (24 per SM instead of 16: 3 % slower), so the instruction count is what is
+// left.  2^24 mixed matrices (10 % of them near-diagonal, on the FP64 path):
+// 2.07 ms, against 6.39 ms when every matrix took the FP64 path (FP64 pipe 83 %
+// busy); eigenvalues only, 10^6: 111 us against 290.
 
 #include <atomic>
 #include <cmath>
@@ -49,6 +51,13 @@ __device__ __forceinline__ int64_t order_key(const double x) {
   return is_zero(x) ? 0 : (b ^ (int64_t)((uint64_t)(b >> 63) >> 1));
 }
 
+// Places in ascending order (equal keys in the order given).
+__device__ __forceinline__ void ranks(const int64_t k0, const int64_t k1, const int64_t k2, int rk[3]) {
+  rk[0] = (int)(k1 < k0) + (int)(k2 < k0);
+  rk[1] = (int)(k0 <= k1) + (int)(k2 < k1);
+  rk[2] = (int)(k0 <= k2) + (int)(k1 <= k2);
+}
+
 // Eigenpairs of an exactly diagonal matrix: the entries and unit vectors, in
 // the order of the arrow reduction (the larger of a11 and a22 first, then the
 // other, a33 last); rk as in fx::solve.
@@ -63,9 +72,7 @@ __device__ __forceinline__ void diagonal(const double a[6], double l[3], double 
   U[1] = U[3] = keep ? 0.0 : 1.0;
   U[2] = U[5] = U[6] = U[7] = 0.0;
   U[8] = 1.0;
-  rk[0] = (int)(k1 < k0) + (int)(k2 < k0);
-  rk[1] = (int)(k0 <= k1) + (int)(k2 < k1);
-  rk[2] = (int)(k0 <= k2) + (int)(k1 <= k2);
+  ranks(k0, k1, k2, rk);
 }
 
 // kVectors = false: eigenvalues only (U_out is NULL).
@@ -101,6 +108,150 @@ struct Shared {
   alignas(8) uint64_t bar[2];
   int n_left, n_hard;
 };
+
+// The FP64 path for the list's last P matrices, one per thread; the whole CTA
+// calls it.  Not inlined: its registers would cost the integer part resident
+// warps.
+template <int kTPB, bool kVectors, bool kServe>
+__device__ __noinline__ void fp64_pass(Shared<kTPB, kServe>& S, const int n_left, const int P, double* lam_out,
+                                       double* U_out, unsigned long long* counters) {
+  const int tid = threadIdx.x, lane_id = tid & 31;
+  const unsigned lt_mask = (1u << lane_id) - 1u;
+  Lane L;
+  L.cls = kIdle;
+  const int at = n_left - P + tid;
+  // A result goes straight to memory (over what the tile's write-back put
+  // there, ordered by the barriers in between).
+  auto put = [&](const double lam[3], const double U[9], const int rk[3]) {
+    const int64_t row = S.at[at];
+    double* dl = kServe ? reinterpret_cast<double*>((uintptr_t)row) : lam_out + row * 3;
+    double* dU = kServe ? S.at_U[kServe ? at : 0] : (U_out != nullptr ? U_out + row * 9 : nullptr);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dl[rk[k]] = lam[k];
+    if (kVectors && dU != nullptr) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) dU[i * 3 + rk[k]] = U[i * 3 + k];
+    }
+  };
+  if (tid < P) {
+    const double a[6] = {S.rec[0][at], S.rec[1][at], S.rec[2][at], S.rec[3][at], S.rec[4][at], S.rec[5][at]};
+    double as[6], lam[3], U[9];
+    int e = 0, rk[3];
+    f64::prescale(a, as, e);  // (every listed matrix is finite)
+    if (weakly_coupled(as, lam, U)) {
+      ranks(order_key(lam[0]), order_key(lam[1]), order_key(lam[2]), rk);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) lam[k] = mul_pow2(lam[k], e);
+      put(lam, U, rk);
+    } else {
+      L = make_lane<false>(a);
+    }
+  }
+  // FP32 seeds, then one FP64 step and the stopping test.  Problem 0 is mu
+  // (A - a1 I), problem 1 is nu (P(a2 I - A)P: spikes swapped), Sec. 1.2.
+  const bool reduced = (L.cls == kReduced);
+  double root[2] = {0.0, 0.0};
+  bool hard[2] = {false, false};
+  double ab = 0.0, pb1[2] = {0.0, 0.0}, pb2[2] = {0.0, 0.0}, pg[2] = {0.0, 0.0};
+  if (reduced) {
+    ab = L.a1 - L.a2;
+    const double bb1 = L.b1 * L.b1, bb2 = L.b2 * L.b2;
+    pb1[0] = bb1; pb2[0] = bb2; pg[0] = L.g - L.a1;
+    pb1[1] = bb2; pb2[1] = bb1; pg[1] = L.a2 - L.g;
+    // FP32 can carry the problem when its data are normal FP32 numbers
+    // with room for the products formed from them: spikes^2 >= 2^-120
+    // (a tiny spike gives a root near its own size, 1/x^2 terms up to
+    // ~2^120) and abar >= 2^-100.  An FP32 value that still underflows only
+    // makes the FP64 step more cautious or sends the root to the full
+    // iteration; acceptance is always the FP64 stopping test.
+    const bool fp32_ok = hi_mag(bb1) >= hi_pow2(-120) && hi_mag(bb2) >= hi_pow2(-120) &&
+                         hi_mag(ab) >= hi_pow2(-100);  // (all three >= 0)
+    float sd[2] = {0.f, 0.f};
+    double pc[2] = {0.0, 0.0}, pK[2] = {0.0, 0.0};
+    const float fab = d2f_rn(ab), fb1[2] = {d2f_rn(pb1[0]), d2f_rn(pb1[1])}, fb2[2] = {d2f_rn(pb2[0]), d2f_rn(pb2[1])};
+    if (fp32_ok) {
+      const double rab = rcp64(ab);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        pc[k] = pb2[k] * rab;
+        pK[k] = -pg[k] - pc[k];
+      }
+      const float fg[2] = {d2f_rn(pg[0]), d2f_rn(pg[1])};
+      const float fc[2] = {d2f_rn(pc[0]), d2f_rn(pc[1])}, fK[2] = {d2f_rn(pK[0]), d2f_rn(pK[1])};
+      seed32x2(fab, fb1, fb2, fg, fc, fK, sd);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      double x = f2d_exact(sd[k]);
+      int st = 2;
+      // 2^-900 <= x <= 2^100 (x >= 0): the range finish64 assumes.
+      if (hi_mag(x) >= hi_pow2(-900) && dbits(x) <= dbits(0x1p+100))
+        st = finish64(ab, pb1[k], pb2[k], pg[k], pc[k], pK[k], fab, fb1[k], fb2[k], x);
+      root[k] = (st == 2) ? 0.0 : x;  // 0: restart from Eq. (7)
+      hard[k] = (st != 0);
+    }
+  }
+  // Compact the unfinished roots and finish them with every lane of the
+  // CTA available.
+  int slot[2] = {-1, -1};
+  {
+    const unsigned m0 = __ballot_sync(0xffffffffu, hard[0]);
+    const unsigned m1 = __ballot_sync(0xffffffffu, hard[1]);
+    const int total = __popc(m0) + __popc(m1);
+    int wbase = 0;
+    if (lane_id == 0 && total) wbase = atomicAdd(&S.n_hard, total);
+    wbase = __shfl_sync(0xffffffffu, wbase, 0);
+    if (hard[0]) slot[0] = wbase + __popc(m0 & lt_mask);
+    if (hard[1]) slot[1] = wbase + __popc(m0) + __popc(m1 & lt_mask);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (slot[k] >= 0) {
+        S.hard.x[slot[k]] = root[k];
+        S.hard.ab[slot[k]] = ab;
+        S.hard.b1[slot[k]] = pb1[k];
+        S.hard.b2[slot[k]] = pb2[k];
+        S.hard.g[slot[k]] = pg[k];
+      }
+    }
+  }
+  __syncthreads();
+  const int n_hard = S.n_hard;
+  for (int i = tid; i < n_hard; i += kTPB) {
+    bool cp;
+    int steps;
+    S.hard.x[i] = zero_bg_full(S.hard.ab[i], S.hard.b1[i], S.hard.b2[i], S.hard.g[i], S.hard.x[i], cp, steps);
+    S.hard.capped[i] = cp;
+  }
+  __syncthreads();
+  bool capped = false;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (slot[k] >= 0) {
+      root[k] = S.hard.x[slot[k]];
+      capped |= S.hard.capped[slot[k]];
+    }
+  }
+  if (L.cls != kIdle) {
+    double lam[3], U[9];
+    const int rk[3] = {0, 1, 2};
+    if (kVectors)
+      finish_lane(L, root[0], root[1], lam, U);
+    else
+      finish_values(L, root[0], root[1], lam);
+    put(lam, U, rk);
+  }
+  if (counters != nullptr) {
+    const unsigned cm = __ballot_sync(0xffffffffu, capped);
+    if (lane_id == 0 && cm) atomicAdd(&counters[0], (unsigned long long)__popc(cm));
+  }
+  __syncthreads();  // the list's records have been read
+  if (tid == 0) {
+    S.n_left = n_left - P;
+    S.n_hard = 0;
+  }
+}
 
 template <int kTPB, bool kBulkIn, bool kVectors, bool kServe = false>
 __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __restrict__ A, int64_t n,
@@ -293,125 +444,7 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
     }
     __syncthreads();  // the staging area has been read; it takes the root list now
 
-    // The FP64 path: the list's last P matrices, one per thread.
-    Lane L;
-    L.cls = kIdle;
-    const int at = n_left - P + tid;
-    if (tid < P) {
-      const double a[6] = {S.rec[0][at], S.rec[1][at], S.rec[2][at], S.rec[3][at], S.rec[4][at], S.rec[5][at]};
-      L = make_lane<false>(a);
-    }
-    // FP32 seeds, then one FP64 step and the stopping test.  Problem 0 is mu
-    // (A - a1 I), problem 1 is nu (P(a2 I - A)P: spikes swapped), Sec. 1.2.
-    const bool reduced = (L.cls == kReduced);
-    double root[2] = {0.0, 0.0};
-    bool hard[2] = {false, false};
-    double ab = 0.0, pb1[2] = {0.0, 0.0}, pb2[2] = {0.0, 0.0}, pg[2] = {0.0, 0.0};
-    if (reduced) {
-      ab = L.a1 - L.a2;
-      const double bb1 = L.b1 * L.b1, bb2 = L.b2 * L.b2;
-      pb1[0] = bb1; pb2[0] = bb2; pg[0] = L.g - L.a1;
-      pb1[1] = bb2; pb2[1] = bb1; pg[1] = L.a2 - L.g;
-      // FP32 can carry the problem when its data are normal FP32 numbers
-      // with room for the products formed from them: spikes^2 >= 2^-120
-      // (a tiny spike gives a root near its own size, 1/x^2 terms up to
-      // ~2^120) and abar >= 2^-100.  An FP32 value that still underflows only
-      // makes the FP64 step more cautious or sends the root to the full
-      // iteration; acceptance is always the FP64 stopping test.
-      const bool fp32_ok = hi_mag(bb1) >= hi_pow2(-120) && hi_mag(bb2) >= hi_pow2(-120) &&
-                           hi_mag(ab) >= hi_pow2(-100);  // (all three >= 0)
-      float sd[2] = {0.f, 0.f};
-      double pc[2] = {0.0, 0.0}, pK[2] = {0.0, 0.0};
-      const float fab = d2f_rn(ab), fb1[2] = {d2f_rn(pb1[0]), d2f_rn(pb1[1])}, fb2[2] = {d2f_rn(pb2[0]), d2f_rn(pb2[1])};
-      if (fp32_ok) {
-        const double rab = rcp64(ab);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          pc[k] = pb2[k] * rab;
-          pK[k] = -pg[k] - pc[k];
-        }
-        const float fg[2] = {d2f_rn(pg[0]), d2f_rn(pg[1])};
-        const float fc[2] = {d2f_rn(pc[0]), d2f_rn(pc[1])}, fK[2] = {d2f_rn(pK[0]), d2f_rn(pK[1])};
-        seed32x2(fab, fb1, fb2, fg, fc, fK, sd);
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        double x = f2d_exact(sd[k]);
-        int st = 2;
-        // 2^-900 <= x <= 2^100 (x >= 0): the range finish64 assumes.
-        if (hi_mag(x) >= hi_pow2(-900) && dbits(x) <= dbits(0x1p+100))
-          st = finish64(ab, pb1[k], pb2[k], pg[k], pc[k], pK[k], fab, fb1[k], fb2[k], x);
-        root[k] = (st == 2) ? 0.0 : x;  // 0: restart from Eq. (7)
-        hard[k] = (st != 0);
-      }
-    }
-    // Compact the unfinished roots and finish them with every lane of the
-    // CTA available.
-    int slot[2] = {-1, -1};
-    {
-      const unsigned m0 = __ballot_sync(0xffffffffu, hard[0]);
-      const unsigned m1 = __ballot_sync(0xffffffffu, hard[1]);
-      const int total = __popc(m0) + __popc(m1);
-      int wbase = 0;
-      if (lane_id == 0 && total) wbase = atomicAdd(&S.n_hard, total);
-      wbase = __shfl_sync(0xffffffffu, wbase, 0);
-      if (hard[0]) slot[0] = wbase + __popc(m0 & lt_mask);
-      if (hard[1]) slot[1] = wbase + __popc(m0) + __popc(m1 & lt_mask);
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        if (slot[k] >= 0) {
-          S.hard.x[slot[k]] = root[k];
-          S.hard.ab[slot[k]] = ab;
-          S.hard.b1[slot[k]] = pb1[k];
-          S.hard.b2[slot[k]] = pb2[k];
-          S.hard.g[slot[k]] = pg[k];
-        }
-      }
-    }
-    __syncthreads();
-    const int n_hard = S.n_hard;
-    for (int i = tid; i < n_hard; i += kTPB) {
-      bool cp;
-      int steps;
-      S.hard.x[i] = zero_bg_full(S.hard.ab[i], S.hard.b1[i], S.hard.b2[i], S.hard.g[i], S.hard.x[i], cp, steps);
-      S.hard.capped[i] = cp;
-    }
-    __syncthreads();
-    bool capped = false;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (slot[k] >= 0) {
-        root[k] = S.hard.x[slot[k]];
-        capped |= S.hard.capped[slot[k]];
-      }
-    }
-    // Eigenpairs, straight to memory (over what the tile's write-back put
-    // there, ordered by the barriers in between).
-    if (tid < P) {
-      double lam[3], U[9];
-      if (kVectors)
-        finish_lane(L, root[0], root[1], lam, U);
-      else
-        finish_values(L, root[0], root[1], lam);
-      const int64_t row = S.at[at];
-      double* dl = kServe ? reinterpret_cast<double*>((uintptr_t)row) : lam_out + row * 3;
-      double* dU = kServe ? S.at_U[kServe ? at : 0] : (want_U ? U_out + row * 9 : nullptr);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) dl[k] = lam[k];
-      if (kVectors && dU != nullptr) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) dU[k] = U[k];
-      }
-    }
-    if (counters != nullptr) {
-      const unsigned cm = __ballot_sync(0xffffffffu, capped);
-      if (lane_id == 0 && cm) atomicAdd(&counters[0], (unsigned long long)__popc(cm));
-    }
-    __syncthreads();  // the list's records have been read
-    if (tid == 0) {
-      S.n_left = n_left - P;
-      S.n_hard = 0;
-    }
+    fp64_pass<kTPB, kVectors, kServe>(S, n_left, P, lam_out, U_out, counters);
     if (flush) break;  // at most kTPB - 1 were left by then
   }
 }

@@ -102,3 +102,20 @@ def test_each_matrix_alone(syev3):
     lam_u, U_u = syev3.syev3_batched(buf[1:].view(-1, 6))
     torch.cuda.synchronize()
     assert np.array_equal(lam_u.cpu().numpy(), lam) and np.array_equal(U_u.cpu().numpy(), U)
+
+
+@pytest.mark.parametrize("k", [24, 26, 27, 28, 29, 30, 40, 60])
+def test_weak_coupling(syev3, k):
+    """Nearly diagonal matrices with every coupling 2^-k of the smallest gap,
+    one of them or two of them zero in some, at the border of the route that
+    takes them by perturbation."""
+    rng = np.random.default_rng(1780 + k)
+    n = 6000
+    d = np.stack([np.zeros(n), rng.uniform(1.0, 2.0, n), rng.uniform(3.0, 2000.0, n)], 1)
+    d = rng.permuted(d - rng.uniform(0.0, 3.0, (n, 1)), axis=1)
+    A = np.concatenate([d, 2.0 ** -k * rng.uniform(0.5, 1.0, (n, 3)) * rng.choice([-1.0, 1.0], (n, 3))], 1)
+    A[: n // 3, 3] = 0.0
+    A[: n // 6, 5] = 0.0
+    A *= 10.0 ** rng.uniform(-50.0, 50.0, (n, 1))
+    lam, _ = check(syev3, A)
+    assert np.array_equal(solve(syev3, A, vectors=False)[0], lam)
