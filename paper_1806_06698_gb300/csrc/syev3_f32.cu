@@ -563,23 +563,26 @@ struct FlagList<true> {
 // kComp32 takes 219 us; refined by single warps as soon as 32 had gathered,
 // 295; by FP64 code on a list per tile (the earlier form) 281.
 // kVectors = false (plain mode only): eigenvalues only, U_out NULL.
+// kRows: matrices per thread and tile.
 // kServe: the serving build.  The tiles are those of the
 // device-resident work list `list` (A, n, lam_out and U_out are unused), each
 // with its own input and output rows; a tile's input is bulk-copied from its
 // first 16-byte boundary-aligned record on, or loaded with plain loads when
 // its start is not 16-byte aligned.  The production builds (kServe = false)
 // compile this out.
-template <bool kBulkIn, int kMode, bool kVectors = true, bool kServe = false>
+template <bool kBulkIn, int kMode, bool kVectors = true, bool kServe = false, int kRows = 1>
 __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32 ? 6 : 8))
     k_syev3_f32(const float* __restrict__ A, int64_t n, float* __restrict__ lam_out, float* __restrict__ U_out,
                 unsigned long long* __restrict__ counters, int64_t* __restrict__ flag_list,
                 unsigned long long* __restrict__ flag_count, const ServeList* __restrict__ list) {
   static_assert(!kServe || (kBulkIn && kMode != kDeferred && kVectors), "the serving build is bulk, vectors");
   static_assert(kTPB == kServeTile, "serving tiles are solve tiles");
+  static_assert(kRows == 1 || (kMode == kPlain && !kServe), "longer tiles: production, plain");
   constexpr bool kComp = kMode != kPlain, kList = kMode == kComp32;
-  __shared__ alignas(16) float s_in[2][kTPB * 6];
-  __shared__ alignas(16) float s_lam[kTPB * 3];
-  __shared__ alignas(16) float s_U[kTPB * 9];
+  constexpr int kTile = kTPB * kRows;
+  __shared__ alignas(16) float s_in[2][kTile * 6];
+  __shared__ alignas(16) float s_lam[kTile * 3];
+  __shared__ alignas(16) float s_U[kTile * 9];
   __shared__ alignas(8) uint64_t s_bar[2];
   __shared__ TileRef<float> s_ref[kServe ? 2 : 1];  // serving build: the tile of each buffer
   constexpr int kCap = FlagList<kServe>::kCap;
@@ -587,7 +590,7 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
   __shared__ int s_nflag;
 
   const int tid = threadIdx.x, lane_id = tid & 31;
-  const int64_t n_tiles = kServe ? list->n_tiles : (n + kTPB - 1) / kTPB;
+  const int64_t n_tiles = kServe ? list->n_tiles : (n + kTile - 1) / kTile;
   bool want_U = (U_out != nullptr);
   bool vec_lam = ((reinterpret_cast<uintptr_t>(lam_out) & 15) == 0);
   bool vec_U = want_U && ((reinterpret_cast<uintptr_t>(U_out) & 15) == 0);
@@ -619,8 +622,8 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
       bulk_g2s(s_in[buf], r.src, bytes, &s_bar[buf]);
       return;
     }
-    const int64_t base = tile * kTPB;
-    const int cnt = (int)((n - base) < kTPB ? (n - base) : kTPB);
+    const int64_t base = tile * kTile;
+    const int cnt = (int)((n - base) < kTile ? (n - base) : kTile);
     const uint32_t bytes = ((uint32_t)cnt * 24u) & ~15u;
     mbar_arrive_expect_tx(&s_bar[buf], bytes);
     if (bytes) bulk_g2s(s_in[buf], A + base * 6, bytes, &s_bar[buf]);
@@ -676,8 +679,8 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
   if (kBulkIn && tid == 0 && tile < n_tiles) issue(tile, 0);
 
   for (; tile < n_tiles; tile += gridDim.x, buf ^= 1, seq += kTPB) {
-    const int64_t base = tile * kTPB;
-    int cnt = (int)((n - base) < kTPB ? (n - base) : kTPB);
+    const int64_t base = tile * kTile;
+    int cnt = (int)((n - base) < kTile ? (n - base) : kTile);
     float* lam_tile = lam_out + base * 3;
     float* U_tile = want_U ? U_out + base * 9 : nullptr;
     const int64_t next = tile + gridDim.x;
@@ -715,86 +718,90 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
       __syncthreads();
     }
 
-    Lane32 L;
-    L.cls = kIdle;
-    L.near_defl = false;
-    if (tid < cnt) {
-      const float2* src = reinterpret_cast<const float2*>(&s_in[buf][tid * 6]);
-      const float2 p0 = src[0], p1 = src[1], p2 = src[2];
-      const float a_in[6] = {p0.x, p0.y, p1.x, p1.y, p2.x, p2.y};
-      L = make_lane32<kComp>(a_in);
-    }
-    // The warp's lanes that form eigenpairs (taken where all 32 are together),
-    // which rejoin after the class-specific part of the solve.
-    const unsigned fin_mask = __ballot_sync(0xffffffffu, L.cls != kIdle && L.cls != kNonFin);
-    float root[2];
-    const bool capped = roots_of<kComp>(L, root);
+    // (not unrolled: two copies of the solve would not fit the instruction cache)
+#pragma unroll 1
+    for (int row = tid; row < kTile; row += kTPB) {
+      Lane32 L;
+      L.cls = kIdle;
+      L.near_defl = false;
+      if (row < cnt) {
+        const float2* src = reinterpret_cast<const float2*>(&s_in[buf][row * 6]);
+        const float2 p0 = src[0], p1 = src[1], p2 = src[2];
+        const float a_in[6] = {p0.x, p0.y, p1.x, p1.y, p2.x, p2.y};
+        L = make_lane32<kComp>(a_in);
+      }
+      // The warp's lanes that form eigenpairs (taken where all 32 are together),
+      // which rejoin after the class-specific part of the solve.
+      const unsigned fin_mask = __ballot_sync(0xffffffffu, L.cls != kIdle && L.cls != kNonFin);
+      float root[2];
+      const bool capped = roots_of<kComp>(L, root);
 
-    bool flagged = false, nonfinite = false;
-    int rk[3] = {0, 1, 2};  // rank of each eigenpair (ascending); identity for the other paths
-    if (L.cls != kIdle) {
-      float l[3], U[9];
-      if (L.cls == kNonFin) {
-        nonfinite = true;
-        const float qnan = __int_as_float(0x7fc00000);
+      bool flagged = false, nonfinite = false;
+      int rk[3] = {0, 1, 2};  // rank of each eigenpair (ascending); identity for the other paths
+      if (L.cls != kIdle) {
+        float l[3], U[9];
+        if (L.cls == kNonFin) {
+          nonfinite = true;
+          const float qnan = __int_as_float(0x7fc00000);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) l[k] = qnan;
+          for (int k = 0; k < 3; ++k) l[k] = qnan;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) U[k] = qnan;
-      } else if (!kVectors) {
-        finish32_values(L, root[0], root[1], l, fin_mask);
-        unscale3(l, L.e);
-      } else {
-        finish32(L, root[0], root[1], l, U, rk, fin_mask);
-        if (kComp && L.cls != kDiag) {
-          // the eigenvalues' gaps in ascending order (min, median, max)
-          const float lo = fminf(fminf(l[0], l[1]), l[2]), hi = fmaxf(fmaxf(l[0], l[1]), l[2]);
-          const float md = fmaxf(fminf(l[0], l[1]), fminf(fmaxf(l[0], l[1]), l[2]));
-          const float nrm2 = fmaf(lo, lo, fmaf(md, md, hi * hi));
-          const float gap = fminf(md - lo, hi - md);
-          flagged = capped || L.near_defl || (gap * gap < (kClusterTau * kClusterTau) * nrm2);
+          for (int k = 0; k < 9; ++k) U[k] = qnan;
+        } else if (!kVectors) {
+          finish32_values(L, root[0], root[1], l, fin_mask);
+          unscale3(l, L.e);
+        } else {
+          finish32(L, root[0], root[1], l, U, rk, fin_mask);
+          if (kComp && L.cls != kDiag) {
+            // the eigenvalues' gaps in ascending order (min, median, max)
+            const float lo = fminf(fminf(l[0], l[1]), l[2]), hi = fmaxf(fmaxf(l[0], l[1]), l[2]);
+            const float md = fmaxf(fminf(l[0], l[1]), fminf(fmaxf(l[0], l[1]), l[2]));
+            const float nrm2 = fmaf(lo, lo, fmaf(md, md, hi * hi));
+            const float gap = fminf(md - lo, hi - md);
+            flagged = capped || L.near_defl || (gap * gap < (kClusterTau * kClusterTau) * nrm2);
+          }
+          unscale3(l, L.e);
         }
-        unscale3(l, L.e);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s_lam[row * 3 + rk[k]] = l[k];
+        if (kVectors) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) s_U[row * 9 + i * 3 + rk[k]] = U[i * 3 + k];
+        }
       }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) s_lam[tid * 3 + rk[k]] = l[k];
-      if (kVectors) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-          for (int i = 0; i < 3; ++i) s_U[tid * 9 + i * 3 + rk[k]] = U[i * 3 + k];
-      }
-    }
 
-    if constexpr (kComp) {
-      const unsigned m = __ballot_sync(0xffffffffu, flagged);
-      const int before = __popc(m & ((1u << lane_id) - 1u));
-      if constexpr (kList) {
-        int at = 0;
-        if (lane_id == 0 && m) at = atomicAdd(&s_nflag, __popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0) + before;
-        if (flagged) {
-          if constexpr (kServe)
-            s_list.at[at] =
-                TileRef<float>{s_ref[buf].src + tid * 6, lam_tile + tid * 3, want_U ? U_tile + tid * 9 : nullptr, 1};
-          else
-            s_list.seq[at] = seq;
+      if constexpr (kComp) {
+        const unsigned m = __ballot_sync(0xffffffffu, flagged);
+        const int before = __popc(m & ((1u << lane_id) - 1u));
+        if constexpr (kList) {
+          int at = 0;
+          if (lane_id == 0 && m) at = atomicAdd(&s_nflag, __popc(m));
+          at = __shfl_sync(0xffffffffu, at, 0) + before;
+          if (flagged) {
+            if constexpr (kServe)
+              s_list.at[at] =
+                  TileRef<float>{s_ref[buf].src + tid * 6, lam_tile + tid * 3, want_U ? U_tile + tid * 9 : nullptr, 1};
+            else
+              s_list.seq[at] = seq;
+          }
+        } else {
+          unsigned long long at = 0;
+          if (lane_id == 0 && m) at = atomicAdd(flag_count, (unsigned long long)__popc(m));
+          at = __shfl_sync(0xffffffffu, at, 0);
+          if (flagged) flag_list[at + before] = base + tid;
         }
-      } else {
-        unsigned long long at = 0;
-        if (lane_id == 0 && m) at = atomicAdd(flag_count, (unsigned long long)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (flagged) flag_list[at + before] = base + tid;
       }
-    }
-    if (counters != nullptr) {
-      const unsigned cm = __ballot_sync(0xffffffffu, capped);
-      const unsigned nf = __ballot_sync(0xffffffffu, nonfinite);
-      const unsigned fl = __ballot_sync(0xffffffffu, flagged);
-      if (lane_id == 0) {
-        if (cm) atomicAdd(&counters[0], (unsigned long long)__popc(cm));
-        if (nf) atomicAdd(&counters[1], (unsigned long long)__popc(nf));
-        if (fl) atomicAdd(&counters[2], (unsigned long long)__popc(fl));
+      if (counters != nullptr) {
+        const unsigned cm = __ballot_sync(0xffffffffu, capped);
+        const unsigned nf = __ballot_sync(0xffffffffu, nonfinite);
+        const unsigned fl = __ballot_sync(0xffffffffu, flagged);
+        if (lane_id == 0) {
+          if (cm) atomicAdd(&counters[0], (unsigned long long)__popc(cm));
+          if (nf) atomicAdd(&counters[1], (unsigned long long)__popc(nf));
+          if (fl) atomicAdd(&counters[2], (unsigned long long)__popc(fl));
+        }
       }
     }
     fence_async_shared();
@@ -803,10 +810,10 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
     // A full, aligned tile's rows leave by bulk copy; the staging area is
     // written again only after thread 0 has seen it read (above, before the
     // next tile's barrier).
-    if (cnt == kTPB && vec_lam && (!want_U || vec_U)) {
+    if (cnt == kTile && vec_lam && (!want_U || vec_U)) {
       if (tid == 0) {
-        bulk_s2g(lam_tile, s_lam, kTPB * 12);
-        if (kVectors && want_U) bulk_s2g(U_tile, s_U, kTPB * 36);
+        bulk_s2g(lam_tile, s_lam, kTile * 12);
+        if (kVectors && want_U) bulk_s2g(U_tile, s_U, kTile * 36);
       }
     } else {
       auto store = [&](float* dst, const float* src, const int m, const bool vec) {
@@ -853,25 +860,27 @@ __global__ void __launch_bounds__(kTPB, 5) k_refine_list(const int64_t* __restri
   }
 }
 
-template <bool kBulkIn, int kMode, bool kVectors, bool kServe = false>
+template <bool kBulkIn, int kMode, bool kVectors, bool kServe = false, int kRows = 1>
 int blocks_per_sm_f32() {
   static int cached = -1;
   if (cached < 0) {
     int v = 0;
-    cudaError_t e =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_syev3_f32<kBulkIn, kMode, kVectors, kServe>, kTPB, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &v, k_syev3_f32<kBulkIn, kMode, kVectors, kServe, kRows>, kTPB, 0);
     cached = (e == cudaSuccess && v > 0) ? v : 1;
   }
   return cached;
 }
 
-template <bool kBulkIn, int kMode, bool kVectors = true>
+template <bool kBulkIn, int kMode, bool kVectors = true, int kRows = 1>
 cudaError_t launch(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters, cudaStream_t stream,
                    int sms, int64_t* flag_list = nullptr, unsigned long long* flag_count = nullptr) {
-  const int64_t n_tiles = (n + kTPB - 1) / kTPB;
-  const int64_t resident = (int64_t)sms * blocks_per_sm_f32<kBulkIn, kMode, kVectors>();
+  constexpr int kTile = kTPB * kRows;
+  const int64_t n_tiles = (n + kTile - 1) / kTile;
+  const int64_t resident = (int64_t)sms * blocks_per_sm_f32<kBulkIn, kMode, kVectors, false, kRows>();
   const int grid = (int)(n_tiles < resident ? n_tiles : resident);
-  k_syev3_f32<kBulkIn, kMode, kVectors><<<grid, kTPB, 0, stream>>>(A, n, lam, U, counters, flag_list, flag_count, nullptr);
+  k_syev3_f32<kBulkIn, kMode, kVectors, false, kRows>
+      <<<grid, kTPB, 0, stream>>>(A, n, lam, U, counters, flag_list, flag_count, nullptr);
   return cudaGetLastError();
 }
 
@@ -886,6 +895,13 @@ cudaError_t launch_serve(const ServeList* list, unsigned long long* counters, cu
 
 }  // namespace
 
+// From this size on (five waves of such tiles) the eigenvalues-only kernel
+// takes two matrices per thread and tile: half the barriers, waits and loop
+// overhead per matrix.  2^23 matrices 149 us against 157; 300763 of them 8.0
+// against 7.2 (fewer tiles than CTAs).  With eigenvectors it gains 1 % and is
+// not used.
+constexpr int64_t kTwoRowsMin = (int64_t)1 << 21;
+
 cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool compensated,
                        unsigned long long* counters, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
@@ -898,7 +914,9 @@ cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool com
   if (compensated)
     return bulk ? launch<true, kComp32>(A, n, lam, U, counters, stream, sms)
                 : launch<false, kComp32>(A, n, lam, U, counters, stream, sms);
-  if (bulk && U == nullptr) return launch<true, kPlain, false>(A, n, lam, U, counters, stream, sms);
+  if (bulk && U == nullptr)
+    return n >= kTwoRowsMin ? launch<true, kPlain, false, 2>(A, n, lam, U, counters, stream, sms)
+                            : launch<true, kPlain, false>(A, n, lam, U, counters, stream, sms);
   return bulk ? launch<true, kPlain>(A, n, lam, U, counters, stream, sms)
               : launch<false, kPlain>(A, n, lam, U, counters, stream, sms);
 }

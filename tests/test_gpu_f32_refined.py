@@ -95,3 +95,14 @@ def test_workspace_form(syev3, n, offset):
     assert torch.equal(lam1, lam2) and torch.equal(U1, U2)
     m = len(A)
     check(np.roll(A, -offset, axis=0), lam1[:m], U1[:m])
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 1, 128, 255, 257])
+def test_eigenvalues_only_in_long_tiles(syev3, extra):
+    """The eigenvalues-only kernel on both sides of the size from which it
+    takes longer tiles: those of the full solve, bit for bit."""
+    n = (1 << 21) + extra
+    A = torch.from_numpy(inputs.mixed_fp32(1 << 17, seed=2140)[0]).cuda().repeat(17, 1)[:n]
+    lam_v, _ = syev3.syev3_batched(A)
+    lam_n, U_n = syev3.syev3_batched(A, vectors=False)
+    assert U_n is None and torch.equal(lam_v, lam_n)
