@@ -8,8 +8,9 @@
 // graded or structured entries, three close eigenvalues -- take the method
 // in FP64 (solve_f64.cuh), whose cost is the FP64 pipe's:
 //  * one matrix per thread; tiles of kTPB packed records arrive by 1-D bulk
-//    copy (TMA) into shared memory, double-buffered on two mbarriers, and
-//    leave through shared-memory staging with 16-byte stores;
+//    copy (TMA) into shared memory, double-buffered on two mbarriers, and a
+//    full tile's results leave their staging rows by bulk copy (2^22 mixed
+//    matrices 500 us, 522 with 16-byte stores by all threads);
 //  * matrices left to the FP64 path are gathered from tile to tile and solved
 //    kTPB at a time, so that each of the SM's FP64 units works on full warps
 //    while the SM's other CTA is in the integer part;
@@ -20,12 +21,12 @@
 //    stopping test; the roots that do not pass are compacted with warp ballots
 //    and finished by the full FP64 iteration.
 //
-// Measured (ncu, 2^22 well-separated matrices): 2370 thread instructions per
-// matrix, issue slots 56 % used, the integer and FMA pipes each about 53 %,
-// the FP64 pipe idle; no one unit is full, more resident warps change nothing
+// Measured (ncu, 2^22 well-separated matrices): 2240 thread instructions per
+// matrix, issue slots 54 % used, the integer and FMA pipes each about 51 %,
+// the FP64 pipe 9 %; no one unit is full, more resident warps change nothing
 // (24 per SM instead of 16: 3 % slower), so the instruction count is what is
 // left.  2^24 mixed matrices (10 % of them near-diagonal, on the FP64 path):
-// 2.07 ms, against 6.39 ms when every matrix took the FP64 path (FP64 pipe 83 %
+// 1.98 ms, against 6.39 ms when every matrix took the FP64 path (FP64 pipe 83 %
 // busy); eigenvalues only, 10^6: 111 us against 290.
 
 #include <atomic>
@@ -319,6 +320,7 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
       double* lam_tile = lam_out + base * 3;
       double* U_tile = want_U ? U_out + base * 9 : nullptr;
       const int64_t next = tile + gridDim.x;
+      if (tid == 0) bulk_read_wait();  // the last tile's rows have left the staging area
       if (kBulkIn) {
         if (tid == 0 && next < n_tiles) issue(next, buf ^ 1);
         const bool ok = mbar_wait(&S.bar[buf], (phases >> buf) & 1u);
@@ -407,33 +409,27 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
         const unsigned nf = __ballot_sync(0xffffffffu, nonfinite);
         if (lane_id == 0 && nf) atomicAdd(&counters[1], (unsigned long long)__popc(nf));
       }
+      fence_async_shared();
       __syncthreads();
 
-      // Coalesced write-back of the tile: 16-byte stores where aligned.  The
-      // rows of matrices in the list receive their results later.
-      {
-        double* const dst = lam_tile;
-        const int m = cnt * 3;
-        if (vec_lam) {
-          double2* d2 = reinterpret_cast<double2*>(dst);
-          const double2* s2 = reinterpret_cast<const double2*>(s_lam);
-          for (int i = tid; i < m / 2; i += kTPB) d2[i] = s2[i];
-          if ((m & 1) && tid == 0) dst[m - 1] = s_lam[m - 1];
-        } else {
-          for (int i = tid; i < m; i += kTPB) dst[i] = s_lam[i];
+      // A full, aligned tile's rows leave by bulk copy; the staging area is
+      // written again only after thread 0 has seen it read (above, before the
+      // next tile's barrier).  The rows of matrices in the list receive their
+      // results later.
+      if (cnt == kTPB && vec_lam && (!want_U || vec_U)) {
+        if (tid == 0) {
+          bulk_s2g(lam_tile, s_lam, kTPB * 24);
+          if (kVectors && want_U) bulk_s2g(U_tile, s_U, kTPB * 72);
         }
-      }
-      if (kVectors && want_U) {
-        double* const dst = U_tile;
-        const int m = cnt * 9;
-        if (vec_U) {
-          double2* d2 = reinterpret_cast<double2*>(dst);
-          const double2* s2 = reinterpret_cast<const double2*>(s_U);
-          for (int i = tid; i < m / 2; i += kTPB) d2[i] = s2[i];
-          if ((m & 1) && tid == 0) dst[m - 1] = s_U[m - 1];
-        } else {
-          for (int i = tid; i < m; i += kTPB) dst[i] = s_U[i];
-        }
+      } else {
+        auto store = [&](double* dst, const double* src, const int m, const bool vec) {
+          const int m2 = vec ? m / 2 : 0;
+          for (int i = tid; i < m2; i += kTPB)
+            reinterpret_cast<double2*>(dst)[i] = reinterpret_cast<const double2*>(src)[i];
+          for (int i = 2 * m2 + tid; i < m; i += kTPB) dst[i] = src[i];
+        };
+        store(lam_tile, s_lam, cnt * 3, vec_lam);
+        if (kVectors && want_U) store(U_tile, s_U, cnt * 9, vec_U);
       }
     }
     const int n_left = S.n_left;  // (stable: between the barrier above and the next tile's)
@@ -442,11 +438,13 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
       if (flush) break;
       continue;
     }
+    if (tid == 0) bulk_write_wait();  // the rows below are written after the tiles' own
     __syncthreads();  // the staging area has been read; it takes the root list now
 
     fp64_pass<kTPB, kVectors, kServe>(S, n_left, P, lam_out, U_out, counters);
     if (flush) break;  // at most kTPB - 1 were left by then
   }
+  if (tid == 0) bulk_read_wait();
 }
 
 // Matrices per tile of a batch.  The integer part is 40 KB of straight-line
