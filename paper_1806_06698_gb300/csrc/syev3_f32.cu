@@ -222,41 +222,57 @@ __device__ __forceinline__ void roots_setup32(const Lane32& L, const float ab, f
   g[0] = gg.x; g[1] = gg.y;
 }
 
-// Double-float value of the spectral function at x (FP32 data exact), and
-// one Newton correction x - f/f' with it (Sec. 1.4.2).  Each term is formed
-// as an unevaluated pair (head, low part) without renormalisation, and the
-// terms are added by cascaded summation (Ogita, Rump and Oishi 2005,
-// "Sum2"): the heads with TwoSum, every rounding error and low part in one
-// FP32 sum, so f comes out as if summed in twice the working precision and
-// rounded once.  Data pairs (ab, b1, b2, g, c, K) need not be normalised.
-__device__ __forceinline__ float newton_ff(const F2 ab, const F2 b1, const F2 b2, const F2 g, const F2 c, const F2 K,
-                                          const float x) {
-  const float r1 = rcp32(x);
-  const F2 s0 = two_sum(x, ab.h);
-  const float sh = s0.h, sl = s0.l + ab.l;  // x + ab
-  const float r2 = rcp32(sh);
+// Double-float value of the spectral function at both roots x (FP32 data
+// exact), and one Newton correction x - f/f' with it (Sec. 1.4.2).  Each
+// term is formed as an unevaluated pair (head, low part) without
+// renormalisation, and the terms are added by cascaded summation (Ogita, Rump
+// and Oishi 2005, "Sum2"): the heads with TwoSum, every rounding error and
+// low part in one FP32 sum, so f comes out as if summed in twice the working
+// precision and rounded once.  Data pairs (ab, b1, b2, -g, c, K) need not be
+// normalised.
+__device__ __forceinline__ P2 pneg(const P2 a) { return pmul(a, pp(-1.f)); }
+
+__device__ __forceinline__ void ptwo_sum(const P2 a, const P2 b, P2& s, P2& e) {
+  s = padd(a, b);
+  const P2 bb = psub(s, a);
+  e = padd(psub(a, psub(s, bb)), psub(b, bb));
+}
+
+__device__ __forceinline__ P2 newton_ff2(const P2 abh, const P2 abl, const P2 b1h, const P2 b1l, const P2 b2h,
+                                        const P2 b2l, const P2 ngh, const P2 ngl, const P2 ch, const P2 cl,
+                                        const P2 Kh, const P2 Kl, const P2 x) {
+  const P2 r1 = prcp(x), nx = pneg(x);
+  P2 sh, s0l;
+  ptwo_sum(x, abh, sh, s0l);
+  const P2 sl = padd(s0l, abl);  // x + ab = sh + sl
+  const P2 r2 = prcp(sh);
   // b1 / x: the quotient's head and the remainder over x.
-  const float q1 = b1.h * r1;
-  const float q1l = (fmaf(-q1, x, b1.h) + b1.l) * r1;
-  // Last term: + c x / (x + ab) for x < ab (the cancellation-free form),
-  // - b2 / (x + ab) otherwise; numerator (nh, nl), quotient (q2, q2l).
-  const bool small = x < ab.h;
-  const float cx = c.h * x;
-  const float nh = small ? cx : b2.h;
-  const float nl = small ? fmaf(c.h, x, -cx) + c.l * x : b2.l;
-  const float q2 = nh * r2;
-  const float q2l = ((fmaf(-q2, sh, nh) + nl) - q2 * sl) * r2;
-  const float th = small ? q2 : -q2, tl = small ? q2l : -q2l;
-  // Leading part: K (small) or -g.
-  const float lh = small ? K.h : -g.h, ll = small ? K.l : -g.l;
+  const P2 q1 = pmul(b1h, r1);
+  const P2 q1l = pmul(padd(pfma(q1, nx, b1h), b1l), r1);
+  // Last term: + c x / (x + ab) below ab (the cancellation-free form),
+  // - b2 / (x + ab) above; numerator (nh, nl), quotient (q2, q2l).
+  const bool sx = x.x < abh.x, sy = x.y < abh.y;
+  const P2 cx = pmul(ch, x);
+  const P2 nh = psel(sx, sy, cx, b2h);
+  const P2 nl = psel(sx, sy, pfma(cl, x, pfma(ch, x, pneg(cx))), b2l);
+  const P2 q2 = pmul(nh, r2), nq2 = pneg(q2);
+  const P2 q2l = pmul(pfma(nq2, sl, padd(pfma(nq2, sh, nh), nl)), r2);
+  const P2 sg = psel(sx, sy, pp(1.f), pp(-1.f));
+  const P2 th = pmul(q2, sg), tl = pmul(q2l, sg);
+  const P2 lh = psel(sx, sy, Kh, ngh), ll = psel(sx, sy, Kl, ngl);
   // Sum2 over x + lead - b1/x + last.
-  const F2 u = two_sum(x, lh);
-  const F2 v = two_sum(u.h, -q1);
-  const F2 w = two_sum(v.h, th);
-  const float f = w.h + (((u.l + v.l) + (w.l + ll)) + (tl - q1l));
-  const float fp = fmaf(b2.h * r2, r2, fmaf(q1, r1, 1.f));
-  const float xn = x - f * rcp32(fp);
-  return (xn > 0.f) ? xn : x;
+  P2 uh, ul, vh, vl, wh, wl;
+  ptwo_sum(x, lh, uh, ul);
+  vh = psub(uh, q1);  // TwoSum(u.h, -q1)
+  {
+    const P2 bb = psub(vh, uh);
+    vl = psub(psub(uh, psub(vh, bb)), padd(q1, bb));
+  }
+  ptwo_sum(vh, th, wh, wl);
+  const P2 f = padd(wh, padd(padd(padd(ul, vl), padd(wl, ll)), psub(tl, q1l)));
+  const P2 fp = pfma(pmul(b2h, r2), r2, pfma(q1, r1, pp(1.f)));
+  const P2 xn = pfma(pneg(f), prcp(fp), x);
+  return psel(xn.x > 0.f, xn.y > 0.f, xn, x);
 }
 
 // The roots (Sec. 1.2) of a lane: root[0] = mu, root[1] = nu (0 for the other
@@ -289,24 +305,25 @@ __device__ __forceinline__ bool roots_of(const Lane32& L, float root[2]) {
   }
   if (kComp && L.cls == kRed) {
     // Exact FP32 data as double-float, then one Newton correction with a
-    // double-float f at each root.
+    // double-float f at each root (both problems paired).
     const F2 abf = two_sum(L.a1, -L.a2);
-    const float rabh = rcp32(abf.h);
-    const F2 fb1 = two_prod(L.b1, L.b1), fb2 = two_prod(L.b2, L.b2);
-    const F2 fg0 = two_sum(L.g, -L.a1), fg1 = two_sum(L.a2, -L.g);
+    const P2 abh = pp(abf.h), abl = pp(abf.l), rabh = pp(rcp32(abf.h));
+    // spikes (b1^2, b2^2) exactly; problem 1 has them swapped
+    const P2 Bs = make_float2(L.b1, L.b2);
+    const P2 bh = pmul(Bs, Bs), bl = pfma(Bs, Bs, pneg(bh));
+    const P2 sbh = make_float2(bh.y, bh.x), sbl = make_float2(bl.y, bl.x);
+    P2 gh, gl;  // (g - a1, a2 - g) exactly
+    ptwo_sum(make_float2(L.g, L.a2), make_float2(-L.a1, -L.g), gh, gl);
     // c = b2 / abar and K = -(g + c) as unnormalised pairs.
-    auto div_pair = [rabh, abf](const F2 num) {
-      const float q = num.h * rabh;
-      return F2{q, ((fmaf(-q, abf.h, num.h) + num.l) - q * abf.l) * rabh};
-    };
-    auto neg_sum_pair = [](const F2 a, const F2 b) {
-      const F2 t = two_sum(a.h, b.h);
-      return F2{-t.h, -((t.l + a.l) + b.l)};
-    };
-    const F2 fc0 = div_pair(fb2), fc1 = div_pair(fb1);
-    const F2 fK0 = neg_sum_pair(fg0, fc0), fK1 = neg_sum_pair(fg1, fc1);
-    root[0] = newton_ff(abf, fb1, fb2, fg0, fc0, fK0, root[0]);
-    root[1] = newton_ff(abf, fb2, fb1, fg1, fc1, fK1, root[1]);
+    const P2 ch = pmul(sbh, rabh);
+    const P2 cl = pmul(pfma(pneg(ch), abl, padd(pfma(pneg(ch), abh, sbh), sbl)), rabh);
+    P2 th, tl;
+    ptwo_sum(gh, ch, th, tl);
+    const P2 Kh = pneg(th), Kl = pneg(padd(padd(tl, gl), cl));
+    const P2 xr = newton_ff2(abh, abl, bh, bl, sbh, sbl, pneg(gh), pneg(gl), ch, cl, Kh, Kl,
+                             make_float2(root[0], root[1]));
+    root[0] = xr.x;
+    root[1] = xr.y;
   }
   return capped;
 }
