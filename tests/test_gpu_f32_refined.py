@@ -106,3 +106,14 @@ def test_eigenvalues_only_in_long_tiles(syev3, extra):
     lam_v, _ = syev3.syev3_batched(A)
     lam_n, U_n = syev3.syev3_batched(A, vectors=False)
     assert U_n is None and torch.equal(lam_v, lam_n)
+
+
+@pytest.mark.parametrize("compensated", [False, True])
+@pytest.mark.parametrize("decades", [2, 6, 12])
+def test_spread_entries(syev3, decades, compensated):
+    """Entries spread over many decades: starts far from the roots, so that
+    lanes take the restart and the steps after the fixed schedule."""
+    rng = np.random.default_rng(2150 + decades)
+    A = (rng.standard_normal((1 << 17, 6)) * 10.0 ** rng.uniform(-decades, 0.0, (1 << 17, 6))).astype(np.float32)
+    lam, U = syev3.syev3_batched(torch.from_numpy(A).cuda(), compensated=compensated)
+    check(A, lam, U)
