@@ -45,6 +45,13 @@ __device__ __forceinline__ float rsqrt32(float x) {
   return y;
 }
 
+// The largest of three magnitudes; NaN if one is NaN.
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(fabsf(c)));
+  return y;
+}
+
 // 2^k for -1022 <= k <= 1023, built from its exponent field.
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 

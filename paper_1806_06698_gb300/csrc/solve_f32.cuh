@@ -24,24 +24,20 @@ struct Rot32 {
 };
 
 __device__ __forceinline__ Rot32 ordered_rotation32(float p, float q, float r) {
+  // (selects, no branch: batches with diagonal matrices would take both sides;
+  // 2^23 mixed matrices 179.9 -> 177.4 us together with the paired pre-scale)
   Rot32 J;
-  if (q == 0.f) {
-    const bool keep = p >= r;
-    J.c = keep ? 1.f : 0.f;
-    J.s = keep ? 0.f : 1.f;
-    J.l1 = keep ? p : r;
-    J.l2 = keep ? r : p;
-    return J;
-  }
   const float D = p - r, q2 = q + q;
   const float rad = sqrt32(fmaf(D, D, q2 * q2));
   const float den = fabsf(D) + rad;
-  const float t = (den > 0.f) ? q2 * rcp32(den) : copysignf(1.f, q);
+  float t = (den > 0.f) ? q2 * rcp32(den) : copysignf(1.f, q);
+  if (q == 0.f) t = 0.f;
   const bool right = D >= 0.f;
   const float hi = right ? p : r, lo = right ? r : p;
   J.l1 = fmaf(t, q, hi);
   J.l2 = fmaf(-t, q, lo);
-  const float k = rsqrt32(fmaf(t, t, 1.f));
+  float k = rsqrt32(fmaf(t, t, 1.f));
+  if (q == 0.f) k = 1.f;
   J.c = right ? k : t * k;
   J.s = right ? t * k : k;
   return J;

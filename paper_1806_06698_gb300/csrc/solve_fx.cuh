@@ -408,9 +408,10 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   // (the last comparison fails for a NaN among the w, which the maxima drop)
   if (!(off <= kOffMax && big <= kRotMax && second <= kSecond && w01 + w02 + w12 < 1.f)) return false;
   // B is of A/2: at 2^60 its diagonal is the eigenvalues'.
-  rk[0] = (int)(B[2] < B[0]) + (int)(B[5] < B[0]);
-  rk[1] = (int)(B[0] <= B[2]) + (int)(B[5] < B[2]);
-  rk[2] = (int)(B[0] <= B[5]) + (int)(B[2] <= B[5]);
+  const int b10 = B[2] < B[0], b20 = B[5] < B[0], b21 = B[5] < B[2];
+  rk[0] = b10 + b20;
+  rk[1] = 1 - b10 + b21;
+  rk[2] = 2 - b20 - b21;
   // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
   // and, with the perturbation below, R by 1 + eta.
   const int eta = (int)((N - (1ll << 60)) >> 3);                    // x 2^57

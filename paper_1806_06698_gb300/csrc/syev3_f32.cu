@@ -94,9 +94,10 @@ template <bool kComp>
 __device__ __forceinline__ Lane32 make_lane32(const float a_in[6]) {
   Lane32 L;
   L.near_defl = false;
-  unsigned mag = 0u;  // largest |a_ij| as a bit pattern (orders like |a_ij|)
-#pragma unroll
-  for (int i = 0; i < 6; ++i) mag = max(mag, __float_as_uint(a_in[i]) & 0x7fffffffu);
+  // largest |a_ij| as a bit pattern, NaN above all (3 instructions; by integer
+  // maxima 11, 1.3 % of the kernel together with the ranks of finish32)
+  const unsigned mag = __float_as_uint(
+      max_abs3(max_abs3(a_in[0], a_in[1], a_in[2]), max_abs3(a_in[3], a_in[4], a_in[5]), 0.f));
   if (mag >= 0x7f800000u) {  // an infinite or NaN entry
     L.cls = kNonFin;
     return L;
@@ -107,7 +108,11 @@ __device__ __forceinline__ Lane32 make_lane32(const float a_in[6]) {
     L.e = E - 126;
     const float sc = pow2f(-L.e);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) a[i] = a_in[i] * sc;
+    for (int i = 0; i < 6; i += 2) {
+      const P2 y = pmul(make_float2(a_in[i], a_in[i + 1]), pp(sc));
+      a[i] = y.x;
+      a[i + 1] = y.y;
+    }
   } else {
     float amax = 0.f;
 #pragma unroll
@@ -335,8 +340,6 @@ __device__ __forceinline__ unsigned sign_of_largest(const float y0, const float 
   return __float_as_uint(big) & 0x80000000u;
 }
 
-// Eigenpairs of a classified lane in FP32 (scaled frame); returns eigenvalues
-// ascending in l[] and vectors as columns in U[i*3+k].
 // Eigenvalues only: those of finish32 (the same expressions, compare order
 // and tie rule), ascending, in the scaled frame.
 __device__ __forceinline__ void finish32_values(const Lane32& L, float mu, float nu, float l_out[3],
@@ -365,58 +368,63 @@ __device__ __forceinline__ void finish32_values(const Lane32& L, float mu, float
   l_out[0] = l0; l_out[1] = l1; l_out[2] = l2;
 }
 
+// Eigenpairs of a classified lane in FP32 (scaled frame): eigenvalues in
+// l_out[], vectors as columns in U[i*3+k], their ascending ranks in rk[].  The
+// kernel is bound by instruction issue, so the vectors 0 and 2 are formed in
+// pairs (2^23 mixed matrices 183.5 -> 179.9 us).
 __device__ __forceinline__ void finish32(const Lane32& L, float mu, float nu, float l_out[3], float U[9], int rk[3],
                                          const unsigned sync_mask) {
   const float a1 = L.a1, a2 = L.a2, b1 = L.b1, b2 = L.b2, g = L.g;
-  float l[3], v[3][3];
+  float l[3], v1[3];
+  P2 w[3];  // components of the vectors 0 (.x) and 2 (.y)
   if (L.cls == kDiag) {
     l[0] = a1; l[1] = a2; l[2] = g;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) v[k][i] = (i == k) ? 1.f : 0.f;
+    w[0] = make_float2(1.f, 0.f); w[1] = make_float2(0.f, 0.f); w[2] = make_float2(0.f, 1.f);
+    v1[0] = 0.f; v1[1] = 1.f; v1[2] = 0.f;
   } else if (L.cls == kDefl) {
     const float h2 = fmaf(b1, b1, b2 * b2);
     const float rh = rsqrt32(h2), h = h2 * rh;
     const float gs = b1 * rh, gc = b2 * rh;
     l[0] = fmaf(a1 * gc, gc, a2 * gs * gs);
-    v[0][0] = gc; v[0][1] = -gs; v[0][2] = 0.f;
     const float d2 = fmaf(a1 * gs, gs, a2 * gc * gc);
     const Rot32 K = ordered_rotation32(d2, h, g);
     l[1] = K.l1; l[2] = K.l2;
-    v[1][0] = gs * K.c;  v[1][1] = gc * K.c;  v[1][2] = K.s;
-    v[2][0] = -gs * K.s; v[2][1] = -gc * K.s; v[2][2] = K.c;
+    v1[0] = gs * K.c; v1[1] = gc * K.c; v1[2] = K.s;
+    w[0] = make_float2(gc, -gs * K.s); w[1] = make_float2(-gs, -gc * K.s); w[2] = make_float2(0.f, K.c);
   } else {
-    const float abar = a1 - a2;
     l[0] = a1 + mu;
     l[1] = (nu - mu) + g;
     l[2] = a2 - nu;
-    const float mpa = mu + abar, npa = nu + abar;
-    v[0][0] = b1 * mpa; v[0][1] = b2 * mu;  v[0][2] = mu * mpa;
-    v[2][0] = b1 * nu;  v[2][1] = b2 * npa; v[2][2] = -(nu * npa);
-    v[1][0] = v[1][1] = v[1][2] = 0.f;  // u2 = u1 x u3, formed below in the input frame
+    const P2 r = make_float2(mu, nu), pa = padd(r, pp(a1 - a2));
+    w[0] = pmul(pp(b1), make_float2(pa.x, r.y));
+    w[1] = pmul(pp(b2), make_float2(r.x, pa.y));
+    w[2] = pmul(make_float2(r.x, -r.y), pa);
+    v1[0] = v1[1] = v1[2] = 0.f;  // u2 = u1 x u3, formed below in the input frame
+    P2 ss = pfma(w[0], w[0], pfma(w[1], w[1], pmul(w[2], w[2])));
+    if (!(fminf(ss.x, ss.y) >= 0x1p-100f)) {  // squares near underflow: exact power-of-two rescale
+      P2 sc = pp(1.f);
+      int E0 = 1, E2 = 1;
 #pragma unroll
-    for (int k = 0; k < 3; k += 2) {
-      float ss = fmaf(v[k][0], v[k][0], fmaf(v[k][1], v[k][1], v[k][2] * v[k][2]));
-      if (!(ss >= 0x1p-100f)) {  // squares near underflow: exact power-of-two rescale
-        int E = 1;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) E = max(E, (__float_as_int(v[k][i]) >> 23) & 0xff);
-        const float sc = pow2f(126 - E);
-        v[k][0] *= sc; v[k][1] *= sc; v[k][2] *= sc;
-        ss = fmaf(v[k][0], v[k][0], fmaf(v[k][1], v[k][1], v[k][2] * v[k][2]));
+      for (int i = 0; i < 3; ++i) {
+        E0 = max(E0, (__float_as_int(w[i].x) >> 23) & 0xff);
+        E2 = max(E2, (__float_as_int(w[i].y) >> 23) & 0xff);
       }
-      const float inv = rsqrt32(ss);
-      v[k][0] *= inv; v[k][1] *= inv; v[k][2] *= inv;
+      if (!(ss.x >= 0x1p-100f)) sc.x = pow2f(126 - E0);
+      if (!(ss.y >= 0x1p-100f)) sc.y = pow2f(126 - E2);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) w[i] = pmul(w[i], sc);
+      ss = pfma(w[0], w[0], pfma(w[1], w[1], pmul(w[2], w[2])));
     }
+    const P2 inv = make_float2(rsqrt32(ss.x), rsqrt32(ss.y));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w[i] = pmul(w[i], inv);
   }
   __syncwarp(sync_mask);  // the three classes' lanes rejoin for the common tail
   float x[3][3];
-#pragma unroll
-  for (int k = 0; k < 3; k += 2) {
-    x[k][0] = fmaf(L.c, v[k][0], -L.s * v[k][1]);
-    x[k][1] = fmaf(L.s, v[k][0], L.c * v[k][1]);
-    x[k][2] = v[k][2];
+  {
+    const P2 c2 = pp(L.c), y0 = pfma(c2, w[0], pmul(pp(-L.s), w[1])), y1 = pfma(pp(L.s), w[0], pmul(c2, w[1]));
+    x[0][0] = y0.x; x[0][1] = y1.x; x[0][2] = w[2].x;
+    x[2][0] = y0.y; x[2][1] = y1.y; x[2][2] = w[2].y;
   }
   if (L.cls == kRed) {
     // u2 is the cross product of u1 and u3 (Sec. 1.3), of the normalised
@@ -426,16 +434,17 @@ __device__ __forceinline__ void finish32(const Lane32& L, float mu, float nu, fl
     x[1][1] = fmaf(x[0][2], x[2][0], -x[0][0] * x[2][2]);
     x[1][2] = fmaf(x[0][0], x[2][1], -x[0][1] * x[2][0]);
   } else {
-    x[1][0] = fmaf(L.c, v[1][0], -L.s * v[1][1]);
-    x[1][1] = fmaf(L.s, v[1][0], L.c * v[1][1]);
-    x[1][2] = v[1][2];
+    x[1][0] = fmaf(L.c, v1[0], -L.s * v1[1]);
+    x[1][1] = fmaf(L.s, v1[0], L.c * v1[1]);
+    x[1][2] = v1[2];
   }
   // Stable ascending ranks of the three eigenvalues (strict "<" for the
   // later index keeps equal values in branch order); the caller stores each
   // eigenpair at its rank.
-  rk[0] = (int)(l[1] < l[0]) + (int)(l[2] < l[0]);
-  rk[1] = (int)(l[0] <= l[1]) + (int)(l[2] < l[1]);
-  rk[2] = (int)(l[0] <= l[2]) + (int)(l[1] <= l[2]);
+  const int p = l[1] < l[0], q = l[2] < l[0], r = l[2] < l[1];
+  rk[0] = p + q;
+  rk[1] = 1 - p + r;
+  rk[2] = 2 - q - r;
   // Sign rule: each vector's largest-magnitude component (the first of
   // equals) made positive, by XOR-ing its sign bits with that component's
   // (never zero: at least 1/sqrt(3) in a unit vector).
