@@ -386,14 +386,9 @@ class Server:
         (no copy); clone them before release if they are to be kept."""
         info = self.query(ticket)
         dt = self._keep[ticket].dtype
-        n = info.n
-        if not info.d_U:
-            return _device_view(info.d_lambda, (n, 3), dt), None
-        # One view over both (the vectors follow the values in the arena), cut
-        # in two by strides: importing a pointer costs 5 us, a cut 1.5.
-        gap = (info.d_U - info.d_lambda) // (8 if dt == torch.float64 else 4)
-        both = _device_view(info.d_lambda, (gap + 9 * n,), dt)
-        return both.as_strided((n, 3), (3, 1), 0), both.as_strided((n, 3, 3), (9, 3, 1), gap)
+        lam = _device_view(info.d_lambda, (info.n, 3), dt)
+        U = _device_view(info.d_U, (info.n, 3, 3), dt) if info.d_U else None
+        return lam, U
 
     def release(self, ticket: int):
         _check(self._lib.syev3_server_release(self._h, ticket), "syev3_server_release")
