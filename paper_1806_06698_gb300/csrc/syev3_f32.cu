@@ -921,12 +921,14 @@ cudaError_t launch_serve(const ServeList* list, unsigned long long* counters, cu
 
 }  // namespace
 
-// From this size on (five waves of such tiles) the eigenvalues-only kernel
-// takes two matrices per thread and tile: half the barriers, waits and loop
-// overhead per matrix.  2^23 matrices 149 us against 157; 300763 of them 8.0
-// against 7.2 (fewer tiles than CTAs).  With eigenvectors it gains 1 % and is
-// not used.
-constexpr int64_t kTwoRowsMin = (int64_t)1 << 21;
+// From these sizes on the plain kernel takes two matrices per thread and tile:
+// half the barriers, waits and loop overhead per matrix, against fewer tiles
+// than keep every CTA busy to the end.  us, two rows against one: eigenvalues
+// only (tensors) 2^23 127 / 139, 2^20 17.7 / 19.4, 2^19 9.8 / 10.4, 300763
+// 7.1 / 6.6; with eigenvectors (mixed), whose tiles then cost shared memory for
+// 9 CTAs per SM instead of 12, 2^23 174.5 / 177.0, 3000001 64.4 / 65.3, 2^21
+// 46.8 / 47.0, 2^20 24.6 / 24.2.
+constexpr int64_t kTwoRowsValues = (int64_t)1 << 19, kTwoRowsVectors = (int64_t)1 << 21;
 
 cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool compensated,
                        unsigned long long* counters, cudaStream_t stream) {
@@ -941,8 +943,9 @@ cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool com
     return bulk ? launch<true, kComp32>(A, n, lam, U, counters, stream, sms)
                 : launch<false, kComp32>(A, n, lam, U, counters, stream, sms);
   if (bulk && U == nullptr)
-    return n >= kTwoRowsMin ? launch<true, kPlain, false, 2>(A, n, lam, U, counters, stream, sms)
+    return n >= kTwoRowsValues ? launch<true, kPlain, false, 2>(A, n, lam, U, counters, stream, sms)
                             : launch<true, kPlain, false>(A, n, lam, U, counters, stream, sms);
+  if (bulk && n >= kTwoRowsVectors) return launch<true, kPlain, true, 2>(A, n, lam, U, counters, stream, sms);
   return bulk ? launch<true, kPlain>(A, n, lam, U, counters, stream, sms)
               : launch<false, kPlain>(A, n, lam, U, counters, stream, sms);
 }

@@ -117,3 +117,18 @@ def test_spread_entries(syev3, decades, compensated):
     A = (rng.standard_normal((1 << 17, 6)) * 10.0 ** rng.uniform(-decades, 0.0, (1 << 17, 6))).astype(np.float32)
     lam, U = syev3.syev3_batched(torch.from_numpy(A).cuda(), compensated=compensated)
     check(A, lam, U)
+
+
+@pytest.mark.parametrize("base,vectors", [(1 << 19, False), (1 << 21, True)])
+@pytest.mark.parametrize("extra", [-1, 0, 1, 129, 255])
+def test_long_tiles_give_the_short_tiles_results(syev3, base, vectors, extra):
+    """Both sides of the sizes from which a tile holds two matrices per thread:
+    the results of the batch solved in short pieces, bit for bit."""
+    n = base + extra
+    A = torch.from_numpy(inputs.mixed_fp32(1 << 17, seed=2160)[0]).cuda().repeat(17, 1)[:n]
+    lam, U = syev3.syev3_batched(A, vectors=vectors)
+    for lo in range(0, n, 1 << 18):
+        part = A[lo:lo + (1 << 18)].contiguous()
+        lam_p, U_p = syev3.syev3_batched(part, vectors=vectors)
+        assert torch.equal(lam[lo:lo + len(part)], lam_p)
+        assert U is None or torch.equal(U[lo:lo + len(part)], U_p)
