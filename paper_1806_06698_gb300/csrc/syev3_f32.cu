@@ -859,17 +859,22 @@ __global__ void __launch_bounds__(kTPB, kMode == kPlain ? 11 : (kMode == kComp32
   if (tid == 0) bulk_read_wait();
 }
 
-// The refinement of the deferred form: the listed matrices, in whole warps.
+// The refinement of the deferred form: the listed matrices, a CTA's warps in
+// step (one barrier a turn): they share the fetches of the refinement's 40 KB
+// of straight-line code, whose fetch is the main stall (the workspace form, 4 %
+// flagged, 2^21 matrices 93.2 -> 90.0 us, 2^23 330.3 -> 327.7; CTAs of 256 and
+// 512 threads: no better, slower).
 __global__ void __launch_bounds__(kTPB, 5) k_refine_list(const int64_t* __restrict__ rows,
                                                          const unsigned long long* __restrict__ count,
                                                          const float* __restrict__ A, float* __restrict__ lam_out,
                                                          float* __restrict__ U_out,
                                                          unsigned long long* __restrict__ counters) {
   const int64_t m = (int64_t)*count;
-  const int lane_id = threadIdx.x & 31;
-  for (int64_t i0 = (int64_t)blockIdx.x * kTPB + (threadIdx.x & ~31u); i0 < m; i0 += (int64_t)gridDim.x * kTPB) {
-    const bool active = i0 + lane_id < m;
-    const int64_t row = rows[active ? i0 + lane_id : m - 1];
+  for (int64_t base = (int64_t)blockIdx.x * kTPB; base < m; base += (int64_t)gridDim.x * kTPB) {
+    __syncthreads();
+    const int64_t i = base + threadIdx.x;
+    const bool active = i < m;
+    const int64_t row = rows[active ? i : m - 1];
     float rec[6], out[12];
 #pragma unroll
     for (int k = 0; k < 6; ++k) rec[k] = A[row * 6 + k];
