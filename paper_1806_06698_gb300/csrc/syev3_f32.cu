@@ -39,7 +39,7 @@
 // staging rows by bulk copy too, so that no thread loads and stores them and
 // one barrier per tile fewer is needed (2^24 mixed matrices, plain: 415 us
 // against 484 with 16-byte stores by all threads).  The plain form moves 72 B
-// per matrix; it is bound by instruction issue (21.9 warp instructions per
+// per matrix; it is bound by instruction issue (17.7 warp instructions per
 // matrix, 72 % of the slots), not by HBM.
 
 #include <cmath>
@@ -586,8 +586,9 @@ struct FlagList<true> {
 // (compensated: they are appended to a list in the caller's workspace, for
 // k_refine_list).  Refining at the end, the SM's warps run in step, which
 // matters for 40 KB of straight-line code: with 4 % of 2^22 matrices flagged
-// kComp32 takes 219 us; refined by single warps as soon as 32 had gathered,
-// 295; by FP64 code on a list per tile (the earlier form) 281.
+// kComp32 took 219 us (191 with the present zero finder); refined by single
+// warps as soon as 32 had gathered, 295; by FP64 code on a list per tile (the
+// earlier form) 281.
 // kVectors = false (plain mode only): eigenvalues only, U_out NULL.
 // kRows: matrices per thread and tile.
 // kServe: the serving build.  The tiles are those of the
@@ -956,12 +957,13 @@ cudaError_t launch_f32(const float* A, int64_t n, float* lam, float* U, bool com
 }
 
 // From this size on the workspace form lists its flagged matrices there and
-// refines them with a second kernel: the solve then needs 64 registers instead
-// of 80 (8 CTAs per SM instead of 6), which pays for the second launch and the
+// refines them with a second kernel: the solve then needs 56 registers instead
+// of 80 (9 CTAs per SM instead of 6), which pays for the second launch and the
 // list.  Measured, us, this form against the single kernel: 2^23 matrices with
-// 4 % flagged 363 / 412, none flagged 258 / 277; 2^21: 97 / 114, 76 / 72; 2^20:
-// 58 / 68, 45 / 42.  (The earlier form, the refinement by FP64 code on a second
-// stream beside the solve: 414 at 2^23.)
+// 4 % flagged 328 / 370, 2^21 90 / 101; when the line was drawn 2^21 97 / 114
+// with 4 % flagged and 76 / 72 with none, 2^20 58 / 68 and 45 / 42.  (The
+// earlier form, the refinement by FP64 code on a second stream beside the
+// solve: 414 at 2^23.)
 constexpr int64_t kDeferMin = (int64_t)1 << 21;
 
 cudaError_t launch_f32c_ws(const float* A, int64_t n, float* lam, float* U, unsigned long long* counters, void* work,
