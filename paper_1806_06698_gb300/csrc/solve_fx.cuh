@@ -15,12 +15,14 @@
 //      exact Jacobi rotation (Golub and Van Loan, Matrix Computations, 8.5)
 //      of the closest pair, first-order perturbation towards the third -- is
 //      formed in FP32 and multiplied into q, now with 30-bit components;
-//   3. B is formed again from the new q.  Its off-diagonal entries are below
+//   3. B is formed again from the new q.  |q|^2 is within 2^-27 of 1 (checked:
+//      an integer quaternion of that length gives a rotation whatever steps
+//      led to it) and B's off-diagonal entries are below
 //      2^-27 (checked), so its diagonal holds the eigenvalues, and first-order
 //      perturbation gives the eigenvectors: R (I + W + W^2/2), orthogonal to
 //      rounding, W_ij = B_ij/(B_jj - B_ii) (Kato, Perturbation Theory for
 //      Linear Operators, ch. 2).
-// A matrix that fails the entry or the off-diagonal check (graded or
+// A matrix that fails the entry check or one of step 3 (graded or
 // structured entries, three close eigenvalues, FP32 roots that did not
 // converge) is left to the FP64 path.  The decision depends on the matrix
 // alone, never on its neighbours in the batch, and every FP32 sum of products
@@ -173,6 +175,14 @@ __device__ __forceinline__ void rotated(const Split a[6], const Split r[9], cons
   B[5] = trace + grow - B[0] - B[2];
 }
 
+// The power of two that brings v's largest component to [1/2, 1).
+__device__ __forceinline__ float largest_to_half(const float v[3]) {
+  int E = 1;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) E = max(E, (__float_as_int(v[i]) >> 23) & 0xff);
+  return pow2f(126 - E);
+}
+
 // The eigenvector frame of a (|a| < 1) by the FP32 method: outer
 // eigenvectors u1 and u3 by their closed forms (or the deflated 2x2 solve),
 // the third axis as their cross product; returned as an unnormalised
@@ -188,7 +198,9 @@ __device__ __forceinline__ QuatF frame32(const float a[6]) {
   const float b1 = fmaf(J.c, a[4], J.s * a[5]), b2 = fmaf(J.c, a[5], -J.s * a[4]);
   const float ab = a1 - a2, bb1 = b1 * b1, bb2 = b2 * b2, h2 = fmaf(b1, b1, bb2);
   float v[3], u[3];
-  if (fabsf(ab * b1 * b2) <= 0x1p-23f * fabsf(a1 + a2) * h2) {  // Sec. 1.1: deflated
+  // Sec. 1.1: deflated; also when a spike is so small that its square could
+  // underflow (the test's right-hand side is 0 for a trace-free block).
+  if (fabsf(ab * b1 * b2) <= 0x1p-23f * fabsf(a1 + a2) * h2 || fminf(fabsf(b1), fabsf(b2)) < 0x1p-60f) {
     const float rh = h2 > 0.f ? rsqrt32(h2) : 0.f, h = h2 * rh;
     const float gs = b1 * rh, gc = h2 > 0.f ? b2 * rh : 1.f;
     const Rot32 K = ordered_rotation32(fmaf(a1 * gs, gs, a2 * gc * gc), h, g);
@@ -204,8 +216,19 @@ __device__ __forceinline__ QuatF frame32(const float a[6]) {
     const float mpa = x[0] + ab, npa = x[1] + ab;
     v[0] = b1 * mpa; v[1] = b2 * x[0]; v[2] = x[0] * mpa;
     u[0] = b1 * x[1]; u[1] = b2 * npa; u[2] = -(x[1] * npa);
-    const float iv = rsqrt32(fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2])));
-    const float iu = rsqrt32(fmaf(u[0], u[0], fmaf(u[1], u[1], u[2] * u[2])));
+    float vv = fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2]));
+    float uu = fmaf(u[0], u[0], fmaf(u[1], u[1], u[2] * u[2]));
+    if (!(fminf(vv, uu) >= 0x1p-100f)) {  // squares near underflow (a small spike and a small abar beside g)
+      const float sv = largest_to_half(v), su = largest_to_half(u);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        v[i] *= sv;
+        u[i] *= su;
+      }
+      vv = fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2]));
+      uu = fmaf(u[0], u[0], fmaf(u[1], u[1], u[2] * u[2]));
+    }
+    const float iv = rsqrt32(vv), iu = rsqrt32(uu);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       v[i] *= iv;
@@ -240,9 +263,10 @@ __device__ __forceinline__ QuatF frame32(const float a[6]) {
 // Step 2's rotation for B = (00 01 11 02 12 22): the closest pair (i, j) by a
 // Jacobi rotation about the third axis k with the couplings to k eliminated
 // to second order, then both towards k to first order; (i, j, k) cyclic.
-// Returns the vector part x 2^30 of the quaternion (1; p).  Only ratios of B
-// enter, so its scale is free.
-__device__ __forceinline__ void small_rotation(const int64_t B[6], int p[3]) {
+// p receives the vector part x 2^30 of the quaternion (1; p).  Only ratios of B
+// enter, so its scale is free.  False for a rotation towards k by more than
+// about a radian, where first order says nothing; |p| <= 1 otherwise.
+__device__ __forceinline__ bool small_rotation(const int64_t B[6], int p[3]) {
   const float e01 = to_float(B[1]), e02 = to_float(B[3]), e12 = to_float(B[4]);
   const float g01 = to_float(B[2] - B[0]), g12 = to_float(B[5] - B[2]), g02 = to_float(B[5] - B[0]);
   const float m01 = fabsf(g01), m12 = fabsf(g12), m02 = fabsf(g02);
@@ -258,11 +282,13 @@ __device__ __forceinline__ void small_rotation(const int64_t B[6], int p[3]) {
   const float h = t * rcp32(1.f + sqrt32(fmaf(t, t, 1.f)));  // tan of half the angle
   const float r = rcp32(fmaf(h, h, 1.f)), c = fmaf(2.f, r, -1.f), s = 2.f * h * r;
   const float oi = fmaf(c, fj, -s * fi) * rj, oj = -fmaf(c, fi, s * fj) * ri;
-  const int pi = __float2int_rn(0x1p29f * fmaf(-h, oj, oi)), pj = __float2int_rn(0x1p29f * fmaf(h, oi, oj));
-  const int pk = __float2int_rn(0x1p30f * h);
+  const float wpi = fmaf(-h, oj, oi), wpj = fmaf(h, oi, oj);
+  const int pi = __float2int_rn(0x1p29f * wpi), pj = __float2int_rn(0x1p29f * wpj);
+  const int pk = __float2int_rn(0x1p30f * h);  // h below 0.42
   p[0] = k2 ? pi : (k0 ? pk : pj);
   p[1] = k2 ? pj : (k0 ? pi : pk);
   p[2] = k2 ? pk : (k0 ? pj : pi);
+  return fmaxf(fabsf(wpi), fabsf(wpj)) <= 1.f;
 }
 
 // q (1; p), the components x 2^30 (|p| <= 1: the result is below 2^31).
@@ -296,6 +322,11 @@ __device__ __forceinline__ Quat normalised(const Quat q) {
   return o;
 }
 
+// Largest |eta|, |q|^2 = 2^60 (1 + eta): what `rotated` and `solve` assume.
+// Rounding leaves up to 2^-28.  A frame that came out NaN is q = 0 in integers:
+// then B's off-diagonal entries are at rounding level too, and only this check
+// refuses it.
+constexpr int64_t kNormMax = 1ll << 33;
 // Largest off-diagonal entry of the second B, 2^-27 (x 2^61); the rounding of
 // q to 30 bits leaves up to 2^-28.
 constexpr float kOffMax = 0x1p34f;
@@ -390,7 +421,7 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   for (int i = 0; i < 9; ++i) Rs[i] = split31(R[i]);
   rotated(As, Rs, trace, N, B);
   int p[3];
-  small_rotation(B, p);
+  if (!small_rotation(B, p)) return false;
   q = normalised(times(q, p));
   rotation(q, R, N);
 #pragma unroll
@@ -405,6 +436,8 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   if (!(fabsf(w12) <= kRotMax) && fabsf(e12) <= kNoise) w12 = 0.f;
   const float big = fmaxf(fabsf(w01), fmaxf(fabsf(w02), fabsf(w12)));
   const float second = fmaxf(fabsf(w01 * e01), fmaxf(fabsf(w02 * e02), fabsf(w12 * e12)));
+  const int64_t eta60 = N - (1ll << 60);
+  if (eta60 > kNormMax || eta60 < -kNormMax) return false;
   // (the last comparison fails for a NaN among the w, which the maxima drop)
   if (!(off <= kOffMax && big <= kRotMax && second <= kSecond && w01 + w02 + w12 < 1.f)) return false;
   // B is of A/2: at 2^60 its diagonal is the eigenvalues'.
@@ -414,7 +447,7 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   rk[2] = 2 - b20 - b21;
   // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
   // and, with the perturbation below, R by 1 + eta.
-  const int eta = (int)((N - (1ll << 60)) >> 3);                    // x 2^57
+  const int eta = (int)(eta60 >> 3);                               // x 2^57
   const int shrink = eta - 3 * (int)(((int64_t)eta * eta) >> 58);  // eta - 3/2 eta^2
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
