@@ -440,20 +440,22 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   if (eta60 > kNormMax || eta60 < -kNormMax) return false;
   // (the last comparison fails for a NaN among the w, which the maxima drop)
   if (!(off <= kOffMax && big <= kRotMax && second <= kSecond && w01 + w02 + w12 < 1.f)) return false;
-  // B is of A/2: at 2^60 its diagonal is the eigenvalues'.
-  const int b10 = B[2] < B[0], b20 = B[5] < B[0], b21 = B[5] < B[2];
+  // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
+  // and, with the perturbation below, R by 1 + eta.  B is of A/2: at 2^60 its
+  // diagonal is the eigenvalues'.
+  const int eta = (int)(eta60 >> 3);                               // x 2^57
+  const int shrink = eta - 3 * (int)(((int64_t)eta * eta) >> 58);  // eta - 3/2 eta^2
+  int64_t b[3] = {B[0], B[2], B[5]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) b[k] -= ((int64_t)(int)(b[k] >> 31) * shrink) >> 25;
+  // The places are those of the values returned: the division truncates, which
+  // can change the order of values that agree to 2^-55 of the largest entry.
+  const int b10 = b[1] < b[0], b20 = b[2] < b[0], b21 = b[2] < b[1];
   rk[0] = b10 + b20;
   rk[1] = 1 - b10 + b21;
   rk[2] = 2 - b20 - b21;
-  // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
-  // and, with the perturbation below, R by 1 + eta.
-  const int eta = (int)(eta60 >> 3);                               // x 2^57
-  const int shrink = eta - 3 * (int)(((int64_t)eta * eta) >> 58);  // eta - 3/2 eta^2
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int64_t b = k == 0 ? B[0] : (k == 1 ? B[2] : B[5]);
-    l[k] = to_double_int<60>(b - (((int64_t)(int)(b >> 31) * shrink) >> 25), F.e);
-  }
+  for (int k = 0; k < 3; ++k) l[k] = to_double_int<60>(b[k], F.e);
   if (kVectors) {
     // R (I + W + W^2/2 - eta), W antisymmetric: orthogonal to third order.  The
     // factors are held x 2^57 when W is small enough, as it is but for close
