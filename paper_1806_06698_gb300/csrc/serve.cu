@@ -505,6 +505,7 @@ __global__ void __launch_bounds__(kCtlThreads) k_serve_complete(DevCtl* ctl, Dev
     __threadfence_system();
     volatile Mailbox* vm = mb;
     vm->n_rec = ctl->n_rec;
+    __threadfence_system();  // a host that reads the round as done then reads its records too
     vm->rounds_done = ctl->rounds;
   }
 }
@@ -663,8 +664,13 @@ void syev3_server_s::run() {
   cudaSetDevice(device);
   std::unique_lock<std::mutex> lk(mu);
   for (;;) {
-    poll_mailbox();
+    // The rounds first, then the records: a round that ends between the two
+    // reads counts as in flight and is seen by the next turn.  In the other order
+    // its completions were left unread with nothing in flight, and a client
+    // waited the 20 ms below for them (one burst of small requests in 2000).
     const uint64_t done_rounds = static_cast<volatile Mailbox*>(mb)->rounds_done;
+    std::atomic_thread_fence(std::memory_order_acquire);
+    poll_mailbox();
     const uint64_t inflight = rounds_launched - done_rounds;
     if (inflight > 0 && error == SYEV3_OK) {
       const cudaError_t e = cudaStreamQuery(stream);
