@@ -5,9 +5,9 @@
 // -> 64 bit product and of a 64-bit addition (measured), so a fixed-point
 // multiply-add on 31-bit limbs (three products) costs a tenth of an FP64 one.
 // Packed doubles of similar size are held in fixed point with 62 fractional
-// bits, and absolute errors of 2^-60 are a hundredth of the FP64 rounding of
-// the eigenvalues.  A matrix whose entries are all within 2^20 of the largest
-// is solved so:
+// bits; the eigenvalues' errors, about 2^-57 of the largest entry, are a tenth of
+// FP64 rounding.  A matrix whose entries are all within 2^20 of the largest is
+// solved so:
 //   1. the method of C. F. Borges (arXiv 1806.06698, Secs. 1-1.4.1) in FP32
 //      gives an approximate eigenvector frame, kept as a quaternion: R(q) is
 //      a rotation whatever the rounding of q, so no orthogonalisation follows;
@@ -326,7 +326,7 @@ __device__ __forceinline__ Quat normalised(const Quat q) {
 // Rounding leaves up to 2^-28.  A frame that came out NaN is q = 0 in integers:
 // then B's off-diagonal entries are at rounding level too, and only this check
 // refuses it.
-constexpr int64_t kNormMax = 1ll << 33;
+constexpr int64_t kNormMax = (1ll << 33) - 4;
 // Largest off-diagonal entry of the second B, 2^-27 (x 2^61); the rounding of
 // q to 30 bits leaves up to 2^-28.
 constexpr float kOffMax = 0x1p34f;
@@ -349,16 +349,42 @@ __device__ __forceinline__ float quotient(const float e, const float g) {
 // when every off-diagonal entry is within 2^20 of the largest entry's exponent
 // and every diagonal one is so or zero (similar), or there is no off-diagonal
 // entry at all (diagonal); neither for a non-finite entry.  Entries within
-// 2^8 are held exactly, smaller ones to 2^-62; wider spreads are left to the
-// FP64 path, which keeps small entries to their own relative accuracy.
+// 2^8 are held exactly, smaller ones to 2^-62.
+//
+// The eigenvalues carry an error of about 2^-57 of the largest entry (rms; 2^-54
+// at most), the vectors one of 2^-58 over the gap, whatever the eigenvalue's size.
+// FP64 arithmetic loses 2^-53, but of the entries that an eigenvalue belongs to:
+// it is the better one for graded matrices (D S D, D diagonal) with small rows.
+// With kGraded (results in FP64) therefore
+//  * with a row below 2^-6, an eigenvalue below 2^-6 is formed again from its
+//    vector and the record without rounding (small_value);
+//  * a matrix with a 2x2 block below 2^-5 and two eigenvalues below 2^-6 is
+//    left to the FP64 path, for the vectors of the pair.
+// Against double-double in a CPU build, relative error of the worst eigenvalue
+// (median) and error of the worst vector (99 %), FP64 path / fixed point without
+// this / with it: (1, d, d) with couplings d = 2^-12 4.9e-16, 3.1e-14, 4.9e-16 and
+// 3e-16, 1e-14, 3e-16; D S D with D = (1, 1, 2^-5) 1.5e-16, 4.9e-15, below 1e-16;
+// (1, 2^-5, 2^-5) 1.5e-16, 7.1e-15, 1.5e-16 and 7e-16, 1e-13, 7e-16; random D over
+// 2^-6 1.7e-16, 3.1e-16, 1.3e-16 and 4e-16, 4e-15, 4e-16; ungraded gaussian entries
+// 2.1e-16, below 1e-16 twice.  The lines are drawn where the fixed-point errors
+// begin to exceed the other's and so that few generic matrices cross them: of
+// well-separated spectra 7e-5 are formed again and 4e-5 go to the FP64 path, whose
+// serial chain doubles the time of a small batch (leaving every entry spread
+// beyond 2^8 to it instead: 2 %).  2^22 matrices: well-separated 439 -> 452 us,
+// mixed 486 -> 507, tensors 440 -> 443, rank two 444 -> 597; eigenvalues only 340 ->
+// 362, 374 -> 396, 340 -> 354, 344 -> 537.
 constexpr unsigned kSpread = 20;
+constexpr unsigned kGradedRow = 6, kGradedBlock = 5;
+constexpr int64_t kSmall = 1ll << 54;  // eigenvalues x 2^60
 
 struct Fixed {
   Split a[6];
   int e;
   bool similar, diagonal, finite;
+  int graded;  // bit 0: a row below 2^-kGradedRow; bit 1: a 2x2 block below 2^-kGradedBlock
 };
 
+template <bool kGraded>
 __device__ __forceinline__ Fixed fixed_of(const double a_in[6]) {
   Fixed F;
   unsigned h[6], l[6], top = 0u;
@@ -397,14 +423,66 @@ __device__ __forceinline__ Fixed fixed_of(const double a_in[6]) {
     F.a[i].l = (int)(y0 & 0x7fffffffu) * sign;
   }
   F.similar = far <= kSpread;
+  if (kGraded) {
+    unsigned m[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) m[i] = h[i] & 0x7fffffffu;
+    const unsigned row = min(min(max(max(m[0], m[3]), m[4]), max(max(m[1], m[3]), m[5])), max(max(m[2], m[4]), m[5]));
+    const unsigned block = min(min(max(max(m[0], m[1]), m[3]), max(max(m[0], m[2]), m[4])), max(max(m[1], m[2]), m[5]));
+    F.graded = (int)(row < top - (kGradedRow << 20)) | (int)(block < top - (kGradedBlock << 20)) << 1;
+  }
   return F;
+}
+
+// An eigenvalue below 2^-6 of the largest entry again, from its vector u (whose
+// sign is free) and the record: u^T A u / u^T u in integers, A u x 2^113 without
+// rounding, the products x 2^116, so to 2^-80 of the largest entry (a vector's
+// error enters squared).  Not inlined and in a loop: few matrices need
+// it, and it is short so that its instructions arrive quickly (a warp here
+// keeps its CTA waiting).
+__device__ __noinline__ double small_value(const double* rec, const int e, const double u0, const double u1,
+                                           const double u2) {
+  const int shift = e + 1022 < 64 ? 256 : 0, E = e + 1022 + shift;  // as fixed_of
+  // 53-bit fraction of x, 0 for a zero
+  auto fraction = [](const double x) {
+    const unsigned h = (unsigned)__double2hiint(x);
+    const int64_t m = (int64_t)((uint64_t)((h & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x));
+    return (h & 0x7ff00000u) == 0u ? 0 : ((int)h < 0 ? -m : m);
+  };
+  auto exponent = [](const double x) { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); };
+  // u x 2^60 (|u| < 2)
+  const int64_t r0 = fraction(u0) << 9 >> min(1024 - exponent(u0), 63),
+                r1 = fraction(u1) << 9 >> min(1024 - exponent(u1), 63),
+                r2 = fraction(u2) << 9 >> min(1024 - exponent(u2), 63);
+  __int128 p = 0, q = 0, n = 0, t = 0;
+#pragma unroll 1
+  for (int i = 0, j = 0; i < 3;) {
+    double x = rec[i == j ? i : i + j + 2];
+    if (shift) x = scalbn_rare(x, shift);
+    t += ((__int128)fraction(x) * (j == 0 ? r0 : (j == 1 ? r1 : r2))) >> min(E - exponent(x), (int)kSpread + 1);
+    if (++j < 3) continue;
+    const int64_t r = i == 0 ? r0 : (i == 1 ? r1 : r2);
+    p += (__int128)r * (int64_t)(t >> 57);
+    q += (__int128)r * ((int64_t)(t >> 25) & 0xffffffffll);
+    n += (__int128)r * r;
+    t = 0;
+    j = 0;
+    ++i;
+  }
+  p += q >> 32;
+  // 61 bits of it, x 2^(60 + s), less u^T u - 1
+  const int64_t top = (int64_t)(p >> 56), excess = (int64_t)(n >> 60) - (1ll << 60);
+  const int s = __clzll((top < 0 ? -top : top) | 1024) - 3;
+  const int64_t w = (int64_t)(p >> (56 - s));
+  return to_double_int<60>(w - (((w >> 30) * excess) >> 30), e - s);
 }
 
 // Eigenvalues l[3] and, with kVectors, eigenvectors U[i*3+k] of a matrix of
 // similar entries, without the sign rule; rk[k] is pair k's place in ascending order.
-// False when they could not be certified.
-template <bool kVectors>
-__device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], int rk[3]) {
+// False when they could not be certified.  rec: its record (kGraded only).
+// (The eigenvalues do not depend on kVectors.)
+template <bool kVectors, bool kGraded>
+__device__ __forceinline__ bool solve(const Fixed& F, const double* rec, double l[3], double U[9], int rk[3]) {
   const Split* const As = F.a;
   float af[6];
 #pragma unroll
@@ -443,11 +521,11 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   // R is (1 + eta) times a rotation, |eta| < 2^-27: B is divided by (1 + eta)^2
   // and, with the perturbation below, R by 1 + eta.  B is of A/2: at 2^60 its
   // diagonal is the eigenvalues'.
-  const int eta = (int)(eta60 >> 3);                               // x 2^57
-  const int shrink = eta - 3 * (int)(((int64_t)eta * eta) >> 58);  // eta - 3/2 eta^2
+  const int eta58 = (int)((eta60 + 2) >> 2), eta = (eta58 + 1) >> 1;               // x 2^58, x 2^57
+  const int shrink = eta58 - (int)((3 * (int64_t)eta * eta + (1ll << 56)) >> 57);  // eta - 3/2 eta^2
   int64_t b[3] = {B[0], B[2], B[5]};
 #pragma unroll
-  for (int k = 0; k < 3; ++k) b[k] -= ((int64_t)(int)(b[k] >> 31) * shrink) >> 25;
+  for (int k = 0; k < 3; ++k) b[k] -= ((int64_t)(int)(b[k] >> 31) * shrink) >> 26;
   // The places are those of the values returned: the division truncates, which
   // can change the order of values that agree to 2^-55 of the largest entry.
   const int b10 = b[1] < b[0], b20 = b[2] < b[0], b21 = b[2] < b[1];
@@ -456,7 +534,14 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
   rk[2] = 2 - b20 - b21;
 #pragma unroll
   for (int k = 0; k < 3; ++k) l[k] = to_double_int<60>(b[k], F.e);
-  if (kVectors) {
+  int small = 0;  // bit k: eigenvalue k is to be formed again
+  if (kGraded && F.graded) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) small |= (int)((uint64_t)(b[k] + kSmall) < (uint64_t)(2 * kSmall)) << k;
+    if ((F.graded & 2) && (small & (small - 1))) return false;
+    if (!(F.graded & 1)) small = 0;
+  }
+  if (kVectors || small) {
     // R (I + W + W^2/2 - eta), W antisymmetric: orthogonal to third order.  The
     // factors are held x 2^57 when W is small enough, as it is but for close
     // pairs, else x 2^53.
@@ -483,6 +568,14 @@ __device__ __forceinline__ bool solve(const Fixed& F, double l[3], double U[9], 
       // a third of the conversions on the otherwise idle FP64 pipe (2^22 mixed
       // matrices 522 us, none 530, two thirds 544)
       U[i * 3 + 2] = to_double<61>((R[3 * i + 2] << 1) + (d2 >> shift));
+    }
+    if (kGraded && small) {
+      if (small & 1) l[0] = small_value(rec, F.e, U[0], U[3], U[6]);
+      if (small & 2) l[1] = small_value(rec, F.e, U[1], U[4], U[7]);
+      if (small & 4) l[2] = small_value(rec, F.e, U[2], U[5], U[8]);
+      rk[0] = (int)(l[1] < l[0]) + (int)(l[2] < l[0]);
+      rk[1] = (int)(l[0] <= l[1]) + (int)(l[2] < l[1]);
+      rk[2] = (int)(l[0] <= l[2]) + (int)(l[1] <= l[2]);
     }
   }
   return true;

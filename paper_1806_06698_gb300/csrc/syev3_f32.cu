@@ -533,8 +533,8 @@ __device__ __noinline__ bool refine_record(const float* rec, const bool active, 
     double a[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) a[k] = f2d_exact(rec[k]);
-    const fx::Fixed F = fx::fixed_of(a);
-    if (F.similar && !F.diagonal && fx::solve<true>(F, lam, U, rk)) {
+    const fx::Fixed F = fx::fixed_of<false>(a);
+    if (F.similar && !F.diagonal && fx::solve<true, false>(F, nullptr, lam, U, rk)) {
       done = true;
       bad = check && residual_fails(rec, lam, U);
     }

@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
         a_in[0] = p0.x; a_in[1] = p0.y; a_in[2] = p1.x; a_in[3] = p1.y; a_in[4] = p2.x; a_in[5] = p2.y;
         double l[3], U[9];
         int rk[3] = {0, 1, 2};
-        const fx::Fixed F = fx::fixed_of(a_in);
+        const fx::Fixed F = fx::fixed_of<true>(a_in);
         if (!F.finite) {
           nonfinite = true;
           const double qnan = __longlong_as_double(0x7ff8000000000000LL);
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
           for (int k = 0; k < 9; ++k) U[k] = qnan;
         } else if (F.diagonal) {
           diagonal(a_in, l, U, rk);
-        } else if (F.similar && fx::solve<kVectors>(F, l, U, rk)) {
+        } else if (F.similar && fx::solve<kVectors, true>(F, &S.in[buf][tid * 6], l, U, rk)) {
           if (kVectors) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) fx::sign_rule(U, k);
