@@ -356,32 +356,36 @@ __device__ __forceinline__ float quotient(const float e, const float g) {
 // FP64 arithmetic loses 2^-53, but of the entries that an eigenvalue belongs to:
 // it is the better one for graded matrices (D S D, D diagonal) with small rows.
 // With kGraded (results in FP64) therefore
+//  * a row or a 2x2 block below 2^-8 of the largest entry, or below 2^-6 beside an
+//    entry that is not within 2^12, leaves the matrix to the FP64 path;
+//  * so do a block below 2^-6 and two eigenvalues below 2^-6, for the vectors of
+//    the pair;
 //  * with a row below 2^-6, an eigenvalue below 2^-6 is formed again from its
-//    vector and the record without rounding (small_value);
-//  * a matrix with a 2x2 block below 2^-5 and two eigenvalues below 2^-6 is
-//    left to the FP64 path, for the vectors of the pair.
+//    vector and the record without rounding (small_value).
 // Against double-double in a CPU build, relative error of the worst eigenvalue
 // (median) and error of the worst vector (99 %), FP64 path / fixed point without
 // this / with it: (1, d, d) with couplings d = 2^-12 4.9e-16, 3.1e-14, 4.9e-16 and
 // 3e-16, 1e-14, 3e-16; D S D with D = (1, 1, 2^-5) 1.5e-16, 4.9e-15, below 1e-16;
 // (1, 2^-5, 2^-5) 1.5e-16, 7.1e-15, 1.5e-16 and 7e-16, 1e-13, 7e-16; random D over
-// 2^-6 1.7e-16, 3.1e-16, 1.3e-16 and 4e-16, 4e-15, 4e-16; ungraded gaussian entries
-// 2.1e-16, below 1e-16 twice.  The lines are drawn where the fixed-point errors
-// begin to exceed the other's and so that few generic matrices cross them: of
-// well-separated spectra 7e-5 are formed again and 4e-5 go to the FP64 path, whose
-// serial chain doubles the time of a small batch (leaving every entry spread
-// beyond 2^8 to it instead: 2 %).  2^22 matrices: well-separated 439 -> 452 us,
-// mixed 486 -> 507, tensors 440 -> 443, rank two 444 -> 597; eigenvalues only 340 ->
-// 362, 374 -> 396, 340 -> 354, 344 -> 537.
+// 2^-6 1.7e-16, 3.1e-16, 1.4e-16 and 4e-16, 4e-15, 4e-16; ungraded gaussian entries
+// 2.1e-16, below 1e-16 twice.  What remains: vectors of a pair at 2^-6 (D = (1,
+// 2^-3, 2^-3)) 4e-15 at 99 %, the FP64 path 7e-16.  The lines are drawn where the
+// fixed-point errors begin to exceed the other's and so that few generic matrices
+// cross them: of well-separated spectra 6e-5 are formed again and 2e-5 more go to
+// the FP64 path, whose serial chain adds 8 us to a small batch (leaving every
+// entry spread beyond 2^8 to it: 2 %).  2^22 matrices, us: well-separated 439 ->
+// 452, mixed 487 -> 503, tensors 440 -> 443, rank two 444 -> 597; eigenvalues only
+// 340 -> 362, 374 -> 394, 340 -> 354, 344 -> 537; entries spread over 2^30, most of
+// which the FP64 path takes again, 1273 -> 1636 (1570 when it took all).
 constexpr unsigned kSpread = 20;
-constexpr unsigned kGradedRow = 6, kGradedBlock = 5;
+constexpr unsigned kWide = 12, kGraded6 = 6, kGraded8 = 8;
 constexpr int64_t kSmall = 1ll << 54;  // eigenvalues x 2^60
 
 struct Fixed {
   Split a[6];
   int e;
   bool similar, diagonal, finite;
-  int graded;  // bit 0: a row below 2^-kGradedRow; bit 1: a 2x2 block below 2^-kGradedBlock
+  int graded;  // bit 0: a row below 2^-6 of the largest entry; bit 1: a 2x2 block
 };
 
 template <bool kGraded>
@@ -429,7 +433,8 @@ __device__ __forceinline__ Fixed fixed_of(const double a_in[6]) {
     for (int i = 0; i < 6; ++i) m[i] = h[i] & 0x7fffffffu;
     const unsigned row = min(min(max(max(m[0], m[3]), m[4]), max(max(m[1], m[3]), m[5])), max(max(m[2], m[4]), m[5]));
     const unsigned block = min(min(max(max(m[0], m[1]), m[3]), max(max(m[0], m[2]), m[4])), max(max(m[1], m[2]), m[5]));
-    F.graded = (int)(row < top - (kGradedRow << 20)) | (int)(block < top - (kGradedBlock << 20)) << 1;
+    F.similar &= min(row, block) >= top - ((far > kWide ? kGraded6 : kGraded8) << 20);
+    F.graded = (int)(row < top - (kGraded6 << 20)) | (int)(block < top - (kGraded6 << 20)) << 1;
   }
   return F;
 }
