@@ -452,10 +452,19 @@ __global__ void __launch_bounds__(kTPB, 512 / kTPB) k_syev3_f64(const double* __
 // run in step: with 2 CTAs of 256 threads "no instruction" stalls fall from
 // 1.7 to 0.4 cycles per issue against 4 CTAs of 128 (2^22 mixed matrices:
 // 679 against 774 us; 512 threads 729, 192 x 3 771, 320 x 2 673 but slower on
-// well-separated ones).  Small batches lose nothing: 20000 matrices take 7.6
-// us, 18.8 before.
-constexpr int kTile = 256;
+// well-separated ones).  While every tile of 64 is resident at once (77824
+// matrices) they are that small: the FP64 units of all SMs then share the
+// matrices left to the FP64 path, which with tiles of 256 kept a quarter of the
+// SMs busy (4096 tridiagonal matrices 20.4 -> 12.9 us), and the integer part
+// gains from fewer warps per SM too (well-separated spectra: 4096 7.0 -> 6.0 us,
+// 65000 19.8 -> 17.8; 10^5 in tiles of 64 would gain nothing more).
+constexpr int kTile = 256, kTileSmall = 64;
 constexpr int kMaxDevices = 64;
+
+cudaError_t device_and_sms(int* dev, int* sms) {
+  const cudaError_t e = cudaGetDevice(dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev);
+}
 
 // Resident CTAs per SM; raises the kernel's shared-memory limit the first
 // time it is asked for on a device.
@@ -481,9 +490,7 @@ template <int kTPB, bool kBulkIn, bool kVectors, bool kServe>
 cudaError_t launch_f64_t(const double* A, int64_t n, double* lam, double* U, unsigned long long* counters,
                          const ServeList* list, cudaStream_t stream) {
   int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = device_and_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
   e = blocks_per_sm_f64<kTPB, kBulkIn, kVectors, kServe>(dev, &per_sm);
   if (e != cudaSuccess) return e;
@@ -505,10 +512,17 @@ cudaError_t launch_f64_serve(const ServeList* list, unsigned long long* counters
 cudaError_t launch_f64(const double* A, int64_t n, double* lam, double* U, unsigned long long* counters,
                        cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
-  if ((reinterpret_cast<uintptr_t>(A) & 15) == 0) {
-    if (U == nullptr) return launch_f64_t<kTile, true, false, false>(A, n, lam, U, counters, nullptr, stream);
-    return launch_f64_t<kTile, true, true, false>(A, n, lam, U, counters, nullptr, stream);
+  const bool bulk = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  int dev = 0, sms = 0;
+  const cudaError_t e = device_and_sms(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  if (n <= (int64_t)sms * (512 / kTileSmall) * kTileSmall) {  // (one wave: the kernel's launch bounds)
+    if (bulk && U == nullptr) return launch_f64_t<kTileSmall, true, false, false>(A, n, lam, U, counters, nullptr, stream);
+    if (bulk) return launch_f64_t<kTileSmall, true, true, false>(A, n, lam, U, counters, nullptr, stream);
+    return launch_f64_t<kTileSmall, false, true, false>(A, n, lam, U, counters, nullptr, stream);
   }
+  if (bulk && U == nullptr) return launch_f64_t<kTile, true, false, false>(A, n, lam, U, counters, nullptr, stream);
+  if (bulk) return launch_f64_t<kTile, true, true, false>(A, n, lam, U, counters, nullptr, stream);
   return launch_f64_t<kTile, false, true, false>(A, n, lam, U, counters, nullptr, stream);
 }
 
