@@ -473,10 +473,12 @@ __device__ __forceinline__ void unscale3(float l[3], int e) {
 }
 
 // The FP64 residual check ||A u - lambda u|| <= 16 eps32 ||A||_F of a refined
-// lane against its input record; true when it fails.
+// lane against its input record; true when it fails, for a vector that is not
+// of unit length (a zero vector has no residual) and for a NaN.
 __device__ __forceinline__ bool residual_fails(const float rec[6], const double lam[3], const double U[9]) {
   const double M[3][3] = {{rec[0], rec[3], rec[4]}, {rec[3], rec[1], rec[5]}, {rec[4], rec[5], rec[2]}};
-  double nA = 0.0, worst = 0.0;
+  double nA = 0.0;
+  bool ok = true;
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -489,9 +491,10 @@ __device__ __forceinline__ bool residual_fails(const float rec[6], const double 
       const double v = fma(M[r][0], U[k], fma(M[r][1], U[3 + k], fma(M[r][2], U[6 + k], -lam[k] * U[r * 3 + k])));
       rr = fma(v, v, rr);
     }
-    worst = fmax(worst, rr);
+    const double excess = fma(U[k], U[k], fma(U[3 + k], U[3 + k], fma(U[6 + k], U[6 + k], -1.0)));
+    ok &= rr <= kResidualTol * kResidualTol * nA && fabs(excess) <= kResidualTol;
   }
-  return !(worst <= kResidualTol * kResidualTol * nA);
+  return !ok;
 }
 
 // FP64 refinement of one flagged lane (compensated form): the arrow and the
