@@ -102,7 +102,10 @@ def _stream(stream) -> int:
     if stream is not None:
         return stream.cuda_stream
     if torch.cuda.is_initialized():
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:  # torch's own names: a version without them takes the public call
+            pass
     return torch.cuda.current_stream().cuda_stream
 
 
