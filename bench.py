@@ -351,7 +351,7 @@ def _fp32_legs(args, dev, stream, barrier, A64_dev):
         lam_ref, _ = syev3.syev3_batched(A_ref, stream=stream)
         lam_ref_h = lam_ref.cpu().numpy()
         nrm_h = np.linalg.norm(lam_ref_h, axis=1)
-        # compensated: syev3_batched_ws (the FP64 refinement as a second
+        # compensated: syev3_batched_ws (the refinement as a second
         # kernel over a list in a workspace); compensated_single_kernel:
         # syev3_batched (the refinement inside the FP32 kernel).
         ws = torch.empty(syev3.workspace_bytes(n, torch.float32, compensated=True), dtype=torch.uint8, device=dev)

@@ -90,7 +90,8 @@ int syev3_batched(const void* A_packed6, int64_t n, void* lambda, void* U, int d
  *                [1] lanes with a non-finite input entry,
  *                [2] lanes refined (SYEV3_F32_COMPENSATED only),
  *                [3] refined lanes whose FP64 residual ||A u - lambda u||
- *                    exceeded 16 eps32 ||A||_F (SYEV3_F32_COMPENSATED only).
+ *                    exceeded 16 eps32 ||A||_F, or with a vector not of unit
+ *                    length (SYEV3_F32_COMPENSATED only).
  *                The caller zeroes them; they accumulate across calls.
  */
 int syev3_batched_ex(const void* A_packed6, int64_t n, void* lambda, void* U, int dtype,

@@ -85,10 +85,10 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 
 // Shared -> global bulk copy, one bulk group per call; dst, src 16-byte
-// aligned, bytes a multiple of 16.  The caller makes the CTA's writes to src
-// visible to it first (fence_async_shared after a barrier of the writers) and
-// waits for the reads of src (bulk_read_wait) before src is written again or
-// the thread ends.
+// aligned, bytes a multiple of 16.  Every thread that wrote to src calls
+// fence_async_shared first, then the CTA a barrier, then one thread this; that
+// thread waits for the reads of src (bulk_read_wait) before src is written
+// again or the thread ends.
 __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst),
                "r"(smem_u32(src)), "r"(bytes)

@@ -7,7 +7,7 @@
 namespace syev3 {
 
 // Counters layout (see syev3_batched_ex): [0] capped, [1] non-finite,
-// [2] refined in FP64, [3] refined lanes failing the FP64 residual check.
+// [2] refined, [3] refined lanes failing the FP64 residual check.
 constexpr int kNumCounters = 4;
 
 cudaError_t launch_f64(const double* A, int64_t n, double* lam, double* U, unsigned long long* counters,

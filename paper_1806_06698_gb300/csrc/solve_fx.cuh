@@ -323,7 +323,7 @@ __device__ __forceinline__ Quat normalised(const Quat q) {
 }
 
 // Largest |eta|, |q|^2 = 2^60 (1 + eta): what `rotated` and `solve` assume.
-// Rounding leaves up to 2^-28.  A frame that came out NaN is q = 0 in integers:
+// Rounding leaves 2^-28 and seldom more.  A frame that came out NaN is q = 0 in integers:
 // then B's off-diagonal entries are at rounding level too, and only this check
 // refuses it.
 constexpr int64_t kNormMax = (1ll << 33) - 4;

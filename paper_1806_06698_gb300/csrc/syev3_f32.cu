@@ -64,7 +64,7 @@ constexpr float kEps32 = 0x1p-23f;
 constexpr float kCDefl32 = 1.0f;          // C of the deflation test (Sec. 1.1)
 constexpr float kCTerm32 = 2.0f;          // C of the stopping rule (Sec. 1.4.1)
 constexpr float kTinySpike32 = 0x1p-60f;  // spikes below this are zeroed (beta-deflation)
-// The lanes refined in FP64 are those FP32 cannot resolve: a deflation test
+// The lanes refined are those FP32 cannot resolve: a deflation test
 // whose two sides lie within a factor kNearDefl of each other (the decision
 // rests on the last bits of the FP32 data), or a relative eigenvalue gap
 // below kClusterTau = one unit of FP32 resolution (the pair's eigenvectors are
@@ -527,7 +527,10 @@ __device__ __forceinline__ bool refine_one(const float f[9], const int code, con
 // arrow and roots, formed again by the FP32 solve's own steps.  out:
 // eigenvalues, then eigenvectors.  Whole warps call it; a lane without work
 // passes active = false.  Not inlined: all kernels then share its code and
-// return the same bits.
+// return the same bits.  In the kernels that call it at their end (80 registers
+// a thread) it and the call need 500 bytes of stack and spill some 350, per
+// refined matrix only: more registers would leave fewer CTAs for the FP32 solve
+// (5 per SM instead of 6: slower over all).
 __device__ __noinline__ bool refine_record(const float* rec, const bool active, const bool check, float out[12]) {
   double lam[3], U[9];
   int rk[3] = {0, 1, 2};
