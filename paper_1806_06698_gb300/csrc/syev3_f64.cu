@@ -21,13 +21,13 @@
 //    stopping test; the roots that do not pass are compacted with warp ballots
 //    and finished by the full FP64 iteration.
 //
-// Measured (ncu, 2^21 well-separated matrices): 2160 thread instructions per
-// matrix, issue slots 54 % used, the integer and FMA pipes each about 51 %,
+// Measured (ncu, 2^21 well-separated matrices): 2240 thread instructions per
+// matrix, issue slots 54 % used, the integer and FMA pipes each about 52 %,
 // the FP64 pipe 9 %; no one unit is full, more resident warps change nothing
 // (24 per SM instead of 16: 3 % slower), so the instruction count is what is
 // left.  2^24 mixed matrices (10 % of them near-diagonal, on the FP64 path):
-// 1.91 ms, against 6.38 ms when every matrix took the FP64 path (FP64 pipe 83 %
-// busy); eigenvalues only, 10^6: 107 us against 287.
+// 1.98 ms, against 6.37 ms when every matrix took the FP64 path (FP64 pipe 83 %
+// busy); eigenvalues only, 10^6: 111 us against 294.
 
 #include <atomic>
 #include <cmath>
